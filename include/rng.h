@@ -166,7 +166,7 @@ int rng_state_words(rng_handle h);
  * evaluation". */
 int rng_generate(rng_handle h, uint64_t n_per_stream, void *out, int fmt);
 /* Few streams with long sequences: when n_streams is too small to fill the
- * device and rows are 32-byte aligned, rng_generate cuts each stream's
+ * device, rng_generate cuts each stream's
  * outputs into segments of 2^l rows (l chosen per kind; gbrng_set_split),
  * starts every segment from the state jumped ahead to it (rng_jump) and
  * runs the segments side by side; the final state goes through a scratch
@@ -175,7 +175,8 @@ int rng_generate(rng_handle h, uint64_t n_per_stream, void *out, int fmt);
  * segment), allocated by the first split call that needs it and grown when
  * a call needs more segments: that call synchronises the device and returns
  * RNG_ERR_OOM if the allocation fails.  A split call captured in a CUDA
- * graph never allocates; it powers the multipliers in the kernel instead.
+ * graph, or whose rows are not 16-byte aligned, never allocates; it powers
+ * the multipliers in the kernel instead.
  * The outputs and the state are those of the plain sequence (sequence
  * splitting, Sec. "Parallelizing RNGs"). */
 

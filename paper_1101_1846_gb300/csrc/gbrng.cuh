@@ -118,6 +118,11 @@ int launch_jump(Gen *g, uint64_t k, cudaStream_t st);
 // segments than it holds (synchronises then; never inside a capture).
 int mwc_jump_table(Gen *g, uint64_t rows, uint64_t segs, cudaStream_t st,
                    const uint64_t **table);
+// The table if it already holds `segs` segments of `rows` rows, else nullptr.
+inline const uint64_t *ready_jump_table(const Gen *g, uint64_t rows, uint64_t segs)
+{
+    return g->jmul_rows == rows && segs <= g->jmul_cap ? g->d_jmul : nullptr;
+}
 // Most segments a split call on a handle of n streams can have.
 uint32_t split_max_segments(uint64_t n);
 

@@ -25,6 +25,8 @@
 //            with 16-byte stores after a warp-shuffle realignment;
 //   tail     the last n % 4 streams, taken by one extra CTA of gen_shift with
 //            4-byte stores.
+// Calls of few streams split into jumped segments: gen_split (aligned rows)
+// or gen_split_shift (the others).
 #pragma once
 
 #include <algorithm>
@@ -89,6 +91,9 @@ gen_shift(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult, uint6
     body_shift<KIND, FMT, HINT>(state, mult, n, steps, out + 4 * g0, ld, s_begin + 4 * g0,
                                 (uint32_t)(left < per_cta ? left : per_cta));
 }
+
+// Warps of groups per CTA of gen_split_shift (249 groups), beside its tail warp.
+constexpr int kShiftSplitWarps = 8;
 
 // Sequence splitting (Sec. "Parallelizing RNGs") for calls with too few
 // streams to fill the device: segment y of the grid produces rows
@@ -207,6 +212,135 @@ gen_split(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult, uint6
 #pragma unroll
             for (int k = 0; k < W; ++k)
                 save4(state + k * n + s0, w[k]);
+            *cnt = 0;
+        }
+    }
+}
+
+// Sequence splitting for rows that are not 16-byte aligned: gen_split's
+// segments and arrival counts with body_shift's realigned rows.  A CTA holds
+// 31K + 1 groups of four streams in K = `warps` warps (one halo lane per warp
+// but the last), the same ones in every segment, and, when count % 4 != 0,
+// one more warp, whose first lanes take the last count % 4 streams in the
+// last CTA of a segment.  A halo lane starts from the same state as its
+// group's owner; the barrier after the loads puts its read before the owner's
+// arrival, so the arrivals of owners and tail lanes (one counter per first
+// stream) cover every read.
+//
+// The row's alignment is uniform over the CTA and chosen at run time, in
+// blocks of four rows (so that xor128's words are renamed, not moved): a
+// compile-time sequence as in gen_shift would double the longest compile
+// and a split call is bound by its jumps, its launch or the write stream.
+// MWC powers are taken in the kernel when the handle's table does not already
+// hold them: this path never allocates and never waits.
+// Split against whole calls on GB300: KISS f32 1001 x 16384 1592 -> 47.9
+// us a call.
+template <int KIND, int FMT, int HINT>
+__global__ void __launch_bounds__(32 * (kShiftSplitWarps + 1))
+gen_split_shift(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult, uint64_t n,
+                uint32_t steps, uint32_t rows, uint32_t *__restrict__ out, uint64_t ld,
+                uint64_t s_begin, uint64_t count, int warps, uint32_t *__restrict__ stash,
+                uint32_t *__restrict__ counters, const uint64_t *__restrict__ jmul, JumpTables T)
+{
+    constexpr int W = KindTraits<KIND>::W;
+    const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
+    const uint64_t main = count & ~(uint64_t)3;
+    const uint32_t per_cta = warps ? 31 * warps + 1 : 0;
+    const uint64_t g0 = (uint64_t)blockIdx.x * per_cta;
+    const uint32_t groups = (uint32_t)min((uint64_t)per_cta, main / 4 - g0);
+    const bool tail_warp = k == warps;  // count % 4 streams, one per lane
+    const uint32_t g = 31u * k + lane;
+    const bool live = tail_warp ? blockIdx.x == gridDim.x - 1 && lane < (int)(count - main)
+                                : g < groups;
+    const bool owner = live && (tail_warp || lane < 31 || k == warps - 1);
+    const bool lead = g == 0;
+    const bool trail = owner && g == groups - 1;
+    const bool prev = live && lane > 0;
+    const bool next = owner && lane < 31 && g + 1 < groups;
+    // the thread's first stream, counted from s_begin, and how many it has
+    const uint64_t c = !live ? 0 : tail_warp ? main + lane : 4 * (g0 + g);
+    const int mine = tail_warp ? 1 : 4;
+    const uint64_t s0 = s_begin + c;
+    const uint32_t segs = gridDim.y, y = blockIdx.y, first = y * rows;
+    const uint32_t n_rows = min(rows, steps - first);
+    uint32_t w[kMaxWords][4] = {};
+    uint32_t a[4] = {};
+    if (live) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {  // a tail lane holds its stream four times
+            const uint64_t s = s0 + (tail_warp ? 0 : i);
+#pragma unroll
+            for (int q = 0; q < W; ++q)
+                w[q][i] = state[q * n + s];
+            if constexpr (KindTraits<KIND>::MULT)
+                a[i] = mult[s];
+        }
+    }
+    __syncthreads();  // halo states are read before any arrival is counted
+    auto save = [&](uint32_t *to) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (i < mine)
+#pragma unroll
+                for (int q = 0; q < W; ++q)
+                    to[q * n + s0 + i] = w[q][i];
+    };
+    uint32_t *cnt = counters + s0;
+    if (owner) {
+        __threadfence();
+        if (atomicAdd(cnt, 1u) == segs) {  // the stash was ready before
+            __threadfence();
+            for (int i = 0; i < mine; ++i)
+                for (int q = 0; q < W; ++q)
+                    state[q * n + s0 + i] = __ldcg(stash + q * n + s0 + i);
+            *cnt = 0;
+        }
+    }
+    if (y > 0 && live) {
+        bool mwc_done = false;
+        if constexpr (KIND == RNG_MWC32 || KIND == RNG_KISS) {
+            if (jmul) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    mwc_apply(__ldg(jmul + (uint64_t)y * n + s0 + (tail_warp ? 0 : i)), a[i],
+                              w[0][i], w[1][i]);
+                mwc_done = true;
+            }
+        }
+        if (mwc_done)
+            jump_streams<KIND, 4, true>(w, a, first, T);
+        else
+            jump_streams<KIND, 4, false>(w, a, first, T);
+    }
+    uint32_t *row = out + (uint64_t)first * ld + c;
+    if (!tail_warp && !live)
+        row = out;  // never stored to; keeps the alignment's arithmetic in range
+    const uint32_t dr = (uint32_t)(ld & 3);
+    uint32_t r = (uint32_t)(((uintptr_t)(out + (uint64_t)first * ld) >> 2) & 3);
+    OutMap m;
+    for (uint32_t j = 0; j < n_rows; j += 4) {
+        if (j % KindTraits<KIND>::SYNC_ROWS == 0)
+            __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (j + q < n_rows) {
+                if (tail_warp) {
+                    const uint32_t o = step_enc<KIND, FMT>(w, a, 0);
+                    if (live)
+                        store4<HINT>(row, o);
+                } else {
+                    shift_row_rt<KIND, FMT, HINT>(w, a, row, r, owner, prev, next, lead, trail, m);
+                }
+            }
+            row += ld;
+            r = (r + dr) & 3u;
+        }
+    }
+    if (y == segs - 1 && owner) {
+        save(stash);
+        __threadfence();
+        if (atomicAdd(cnt, 1u) == segs) {
+            save(state);
             *cnt = 0;
         }
     }
@@ -352,8 +486,34 @@ int launch_kind(int fmt, const GenLaunch &p, cudaStream_t st)
     uint32_t *out = static_cast<uint32_t *>(p.out);
     uint64_t L = 0, S = 0;
     Gen *g = p.owner;
-    if (g && g->d_split && aligned &&
-        split_plan(KIND, count, p.steps, 4, g->jmul_segs, split_fill(false), &L, &S)) {
+    const bool split = g && g->d_split &&
+                       split_plan(KIND, count, p.steps, 4, g->jmul_segs, split_fill(false), &L, &S);
+    if (split && !aligned) {
+        JumpTables T{};
+        int e = needs_jump_tables(KIND) ? jump_tables(&T) : RNG_OK;
+        // a captured call must not keep the table's address: it may grow later
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (!e)
+            e = cuda_status(cudaStreamIsCapturing(st, &cap));
+        if (e)
+            return e;
+        const uint64_t *jmul =
+            cap == cudaStreamCaptureStatusNone ? ready_jump_table(g, L, S) : nullptr;
+        // groups spread evenly over as few CTAs per segment as hold them
+        const uint64_t groups = main / 4, most = 31 * kShiftSplitWarps + 1;
+        const uint64_t few = std::max<uint64_t>((groups + most - 1) / most, 1);
+        const uint64_t per = (groups + few - 1) / few;
+        const int warps = per < 2 ? (int)per : (int)((per - 1 + 30) / 31);
+        const uint64_t tiles = warps ? (groups + 31 * warps) / (31 * warps + 1) : 1;
+        const int threads = 32 * (warps + (count > main ? 1 : 0));
+        auto fn = fmt == RNG_F32 ? gen_split_shift<KIND, RNG_F32, 1>
+                                 : gen_split_shift<KIND, RNG_U32, 1>;
+        fn<<<dim3((unsigned)tiles, (unsigned)S), threads, 0, st>>>(
+            p.state, p.a, p.n, (uint32_t)p.steps, (uint32_t)L, out, p.ld, p.s_begin, count, warps,
+            g->d_split, g->d_cnt, jmul, T);
+        return cuda_status(cudaGetLastError());
+    }
+    if (split) {
         JumpTables T{};
         const uint64_t *jmul = nullptr;
         int e = needs_jump_tables(KIND) ? jump_tables(&T) : RNG_OK;
