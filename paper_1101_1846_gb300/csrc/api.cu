@@ -126,7 +126,12 @@ rng_handle create_range(int kind, uint64_t s_begin, uint64_t n_streams, uint64_t
     g->seed = seed + s_begin;
     g->words = words_of(kind);
     int st = RNG_OK;
-    if (cudaMalloc(&g->d_state, (size_t)g->words * n_streams * 4) != cudaSuccess) {
+    // the kinds with a big GF(2) part keep room for one jump's matrix (32 W
+    // columns of W words) behind the state
+    const size_t state_words = (size_t)g->words * n_streams, at = (state_words + 3) / 4 * 4;
+    const bool cols = kind == RNG_XOR128 || kind == RNG_XORSHIFT8;
+    if (cudaMalloc(&g->d_state, 4 * (cols ? at + 32 * g->words * g->words : state_words)) !=
+        cudaSuccess) {
         st = set_error(RNG_ERR_OOM);
     } else if (has_mult(kind)) {
         // one multiplier per stream, or one packed pair for the base-2^16 kinds
@@ -140,6 +145,8 @@ rng_handle create_range(int kind, uint64_t s_begin, uint64_t n_streams, uint64_t
             st = cuda_status(cudaMemcpy(g->d_a, table + s_begin, n_streams * 4,
                                         cudaMemcpyDeviceToDevice));
     }
+    if (cols && g->d_state)
+        g->d_jump_cols = g->d_state + at;
     // buffers of split calls (few streams only): the final-state stash, the
     // arrival counters (zero) and the MWC jump multipliers
     if (!st && n_streams <= kSplitMaxStreams) {

@@ -24,6 +24,8 @@ struct Gen {
     uint32_t *d_state = nullptr;  // SoA: word w of stream s at d_state[w*n + s]
     uint32_t *d_a = nullptr;      // multipliers (MWC32, KISS), n entries
     cudaStream_t stream = nullptr;
+    uint32_t *d_jump_cols = nullptr;  // RNG_XOR128, RNG_XORSHIFT8: room behind the state
+                                      // for the columns of one rng_jump's matrix
     // Split calls (few streams, long sequences; allocated at creation when
     // n <= kSplitMaxStreams):
     uint32_t *d_split = nullptr;  // final state stash, same layout as d_state

@@ -4,6 +4,7 @@
 // words), of 2^m xorshift32 steps (32 columns) and the affine map (A, C) of
 // 2^m LCG steps.  One CTA builds them on the device by repeated squaring,
 // once per device and process.
+#include <algorithm>
 #include <mutex>
 
 #include "jump.cuh"
@@ -138,16 +139,162 @@ mwc_table_kernel(const uint32_t *__restrict__ a, uint64_t n, uint64_t rows, uint
     out[i] = y == 0 ? 0 : mwc_power(a[s], y * rows);
 }
 
+// rng_jump of the kinds without a big GF(2) part: one stream per thread.
+// KISS and KISS_XOR: the xorshift32 and LCG parts are the same map for every
+// stream.  For more than three set bits of k each CTA composes it first: a
+// stream then takes four table reads in place of 32 columns per set bit (2^20
+// KISS streams by 24 set bits on GB300: 236 -> 105 us, of which the MWC power
+// is 67).  Composing takes a CTA about 2 us, the columns 0.6 us a bit at
+// 76,636 streams (KISS_XOR: 8.7 against 10.1 us at three bits, 9.6 against
+// 10.4 at four, 13.4 against 11.4 at eight).
 template <int KIND>
 __global__ void __launch_bounds__(256) jump_kernel(rng_device_view v, uint64_t k, JumpTables T)
 {
+    constexpr bool kKiss = KIND == RNG_KISS || KIND == RNG_KISS_XOR;
+    __shared__ KissJump J;
+    const bool compose = kKiss && __popcll(k) > 3;
+    if constexpr (kKiss)
+        if (compose)
+            kiss_jump_fill(J, k, T);
     const uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= v.n_streams)
         return;
     Engine<KIND> e;
     e.load(v, s);
-    jump_engine<KIND>(e, k, T);
+    if (!compose) {
+        jump_engine<KIND>(e, k, T);
+    } else if constexpr (KIND == RNG_KISS) {
+        mwc_jump(e.a, e.x, e.c, k);
+        kiss_jump_apply(J, e.y, e.z);
+    } else if constexpr (KIND == RNG_KISS_XOR) {
+        mwc16_jump(e.a & 0xFFFFu, e.z, k);
+        mwc16_jump(e.a >> 16, e.w, k);
+        kiss_jump_apply(J, e.y, e.l);
+    }
     e.store(v, s);
+}
+
+// The columns of M^k (W words each, 32 W of them) for the matrix whose powers
+// M^(2^m) are `table`, one warp per column: out[W j ..] is column j.  The set
+// bits' matrices are copied to shared memory a few at a time, so that a chain
+// of them runs at the reductions' latency.
+template <int W>
+__global__ void __launch_bounds__(128)
+compose_kernel(const uint32_t *__restrict__ table, uint64_t k, uint32_t *__restrict__ out)
+{
+    constexpr int kWords = 32 * W * W, kAtOnce = W == 4 ? 16 : 4;  // 32 KB
+    __shared__ __align__(16) uint32_t level[kAtOnce][kWords];
+    const int lane = threadIdx.x & 31;
+    const int j = blockIdx.x * 4 + (threadIdx.x >> 5);
+    uint32_t v[W];
+#pragma unroll
+    for (int q = 0; q < W; ++q)
+        v[q] = (j >> 5) == q ? 1u << (j & 31) : 0u;
+    for (uint64_t r = k; r;) {
+        int levels = 0;
+        for (; levels < kAtOnce && r; ++levels, r &= r - 1) {
+            const uint32_t *src = table + (size_t)kWords * (__ffsll((long long)r) - 1);
+            for (int i = 4 * threadIdx.x; i < kWords; i += 4 * 128)
+                copy16_async(&level[levels][i], src + i);
+        }
+        copies_done();
+        for (int m = 0; m < levels; ++m)
+            gf2_apply_warp<W>(level[m], v, lane);
+        __syncthreads();
+    }
+    uint32_t mine = 0;
+#pragma unroll
+    for (int q = 0; q < W; ++q)
+        mine = lane == q ? v[q] : mine;
+    if (lane < W)
+        out[W * j + lane] = mine;
+}
+
+// Every stream's W words times the matrix of columns `cols`, by tables of the
+// images of each group of BITS bits (32 W / BITS groups, 2^BITS entries of W
+// words, in shared memory): one read and W xors per group in place of BITS
+// masked columns.  The reads collide like any random 16-byte reads (about 9
+// wavefronts a warp), which is what bounds it; eight-bit groups need 64 KB at
+// W = 4, four-bit groups 32 KB at W = 8.  Measured in
+// launch_jump.
+constexpr int kApplyThreads = 512;
+
+template <int W, int BITS>
+__global__ void __launch_bounds__(kApplyThreads)
+apply_kernel(uint32_t *__restrict__ state, uint64_t n, const uint32_t *__restrict__ cols)
+{
+    constexpr int G = 32 * W / BITS, H = W / 4;
+    extern __shared__ __align__(16) uint4 images[];  // [(G << BITS) * H], then 32 W columns
+    uint4 *const col = images + (G << BITS) * H;
+    for (int i = threadIdx.x; i < 32 * W * H; i += kApplyThreads)
+        col[i] = __ldg(reinterpret_cast<const uint4 *>(cols) + i);
+    __syncthreads();
+    for (int e = threadIdx.x; e < G << BITS; e += kApplyThreads) {
+        uint4 x[H] = {};
+#pragma unroll
+        for (int b = 0; b < BITS; ++b) {
+            const uint32_t mask = 0u - ((uint32_t)(e >> b) & 1u);
+#pragma unroll
+            for (int h = 0; h < H; ++h) {
+                const uint4 c = col[((e >> BITS) * BITS + b) * H + h];
+                x[h].x ^= c.x & mask;
+                x[h].y ^= c.y & mask;
+                x[h].z ^= c.z & mask;
+                x[h].w ^= c.w & mask;
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < H; ++h)
+            images[e * H + h] = x[h];
+    }
+    __syncthreads();
+    for (uint64_t s = (uint64_t)blockIdx.x * kApplyThreads + threadIdx.x; s < n;
+         s += (uint64_t)gridDim.x * kApplyThreads) {
+        uint32_t v[W];
+#pragma unroll
+        for (int q = 0; q < W; ++q)
+            v[q] = state[q * n + s];
+        uint4 x[H] = {};
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            const uint32_t e = (v[g * BITS / 32] >> (g * BITS % 32)) & ((1u << BITS) - 1);
+#pragma unroll
+            for (int h = 0; h < H; ++h) {
+                const uint4 c = images[((g << BITS) + e) * H + h];
+                x[h].x ^= c.x;
+                x[h].y ^= c.y;
+                x[h].z ^= c.z;
+                x[h].w ^= c.w;
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            state[(4 * h) * n + s] = x[h].x;
+            state[(4 * h + 1) * n + s] = x[h].y;
+            state[(4 * h + 2) * n + s] = x[h].z;
+            state[(4 * h + 3) * n + s] = x[h].w;
+        }
+    }
+}
+
+template <int W, int BITS>
+int launch_composed(Gen *g, uint64_t k, const uint32_t *table, cudaStream_t st)
+{
+    constexpr int smem = ((32 * W / BITS << BITS) + 32 * W) * W * 4;
+    int e = cuda_status(cudaFuncSetAttribute(
+        apply_kernel<W, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    if (e)
+        return e;
+    compose_kernel<W><<<8 * W, 128, 0, st>>>(table, k, g->d_jump_cols);
+    e = cuda_status(cudaGetLastError());
+    if (e)
+        return e;
+    // resident CTAs stay and walk the streams: each builds the tables once
+    const uint64_t blocks =
+        std::min<uint64_t>((g->n + kApplyThreads - 1) / kApplyThreads, 152 * (W == 4 ? 3 : 4));
+    apply_kernel<W, BITS>
+        <<<(unsigned)blocks, kApplyThreads, smem, st>>>(g->d_state, g->n, g->d_jump_cols);
+    return cuda_status(cudaGetLastError());
 }
 
 }  // namespace
@@ -233,6 +380,15 @@ int launch_jump(Gen *g, uint64_t k, cudaStream_t stream)
         if (st)
             return st;
     }
+    // The kinds with a big GF(2) part multiply the set bits' matrices together
+    // first, also for a single bit: 2^20 streams jumped by 24 set bits (GB300,
+    // us a call, before -> after) xor128 1305 -> 29, XORSHIFT8 5627 -> 165; 256
+    // streams by one set bit 8.4 -> 5.1 and 25.4 -> 9.2, by 24 bits 178 -> 7.5
+    // and 577 -> 20.
+    if (g->kind == RNG_XOR128)
+        return launch_composed<4, 8>(g, k, reinterpret_cast<const uint32_t *>(T.xor128), stream);
+    if (g->kind == RNG_XORSHIFT8)
+        return launch_composed<8, 4>(g, k, reinterpret_cast<const uint32_t *>(T.xs8), stream);
     rng_device_view v{g->kind, g->device, g->words, g->n, g->d_state, g->d_a};
     const uint64_t blocks = (g->n + 255) / 256;
     if (blocks > 0x7FFFFFFFull)
@@ -240,10 +396,8 @@ int launch_jump(Gen *g, uint64_t k, cudaStream_t stream)
     const unsigned b = (unsigned)blocks;
     switch (g->kind) {
     case RNG_MWC32: jump_kernel<RNG_MWC32><<<b, 256, 0, stream>>>(v, k, T); break;
-    case RNG_XOR128: jump_kernel<RNG_XOR128><<<b, 256, 0, stream>>>(v, k, T); break;
     case RNG_KISS: jump_kernel<RNG_KISS><<<b, 256, 0, stream>>>(v, k, T); break;
     case RNG_MWC16X2: jump_kernel<RNG_MWC16X2><<<b, 256, 0, stream>>>(v, k, T); break;
-    case RNG_XORSHIFT8: jump_kernel<RNG_XORSHIFT8><<<b, 256, 0, stream>>>(v, k, T); break;
     default: jump_kernel<RNG_KISS_XOR><<<b, 256, 0, stream>>>(v, k, T); break;
     }
     return cuda_status(cudaGetLastError());
