@@ -19,36 +19,116 @@ namespace {
 
 constexpr int kThreads = 256;
 
-// The sums run in chunks of up to 2^30 outputs with a 32-bit counter and an
-// unroll of 32: loop bookkeeping then costs little beside the step (the MWC
-// sum measured 11 % faster on GB300 than with a 64-bit counter and an
-// unroll of 8; the other kinds were unchanged).
+// The next output.  MWC32 steps by a wide product and two carrying adds here:
+// that takes the adds off the FMA-heavy pipe, which bounds its consumers
+// (2^22 x 1024 on GB300: sum_u32 810 -> 699 us a call, disc 1029 -> 934), where
+// KISS, whose ALU pipe is as full, would lose 2-5 % by it.
+template <int KIND>
+__device__ __forceinline__ uint32_t next_of(Engine<KIND> &e)
+{
+    if constexpr (KIND == RNG_MWC32) {
+        uint32_t lo, hi;
+        asm("{\n\t.reg .u64 q;\n\t.reg .u32 l, h;\n\t"
+            "mul.wide.u32 q, %2, %3;\n\t"
+            "mov.b64 {l, h}, q;\n\t"
+            "add.cc.u32 %0, l, %4;\n\t"
+            "addc.u32 %1, h, 0;\n\t}"
+            : "=r"(lo), "=r"(hi)
+            : "r"(e.a), "r"(e.x), "r"(e.c));
+        e.x = lo;
+        e.c = hi;
+        return lo;
+    } else {
+        return e.next();
+    }
+}
+
+// A pair (u0, u1) is inside when X^2 + Y^2 < 2^48, X = u0 >> 8, Y = u1 >> 8.
+template <int KIND>
+__device__ __forceinline__ uint32_t disc_pair(Engine<KIND> &e)
+{
+    const uint64_t X = next_of(e) >> 8;
+    const uint64_t Y = next_of(e) >> 8;
+    return (X * X + Y * Y) >> 48 == 0 ? 1u : 0u;
+}
+
+// kPairs pairs, counted exactly, mostly in FP32.  With f0, f1 the outputs
+// rounded to FP32 (no shift), d = f0^2 + (f1^2 - 2^64) is off
+// (256 X)^2 + (256 Y)^2 - 2^64 by less than 2^43: f0 is off 256 X by at most
+// 255 + 128, hence its square by 383 x 2^33, twice, and the two roundings by
+// 2^39 each.  So d's sign decides where |d| >= 2^43, and a block with a
+// smaller |d| (16 pi/4 2^-20: one in 83,000 of a thread's blocks) is counted
+// again in integers from the state it began with.
+// The integer test's two wide multiply-adds share the FMA-heavy pipe with the
+// MWC and LCG steps; the conversions, the sign's add and the minimum run on
+// the ALU pipe and the FP32 multiply-adds on either half of the FMA pipe.
+// 2^22 x 1024 on GB300, us a call, integer test -> this: MWC 1385 -> 1029 (934
+// with next_of's step), xor128 2164 -> 1580, KISS 2323 -> 1967.
+constexpr int kPairs = 16;
+
+template <int KIND>
+__device__ __forceinline__ uint32_t disc_block(Engine<KIND> &e)
+{
+    const Engine<KIND> begin = e;
+    uint32_t inside = 0;
+    float least = 0x1p64f;
+#pragma unroll
+    for (int j = 0; j < kPairs; ++j) {
+        const float f0 = __uint2float_rn(next_of(e));
+        const float f1 = __uint2float_rn(next_of(e));
+        const float d = __fmaf_rn(f0, f0, __fmaf_rn(f1, f1, -0x1p64f));
+        inside += __float_as_uint(d) >> 31;
+        least = fminf(least, fabsf(d));
+    }
+    if (least < 0x1p43f) {
+        e = begin;
+        inside = 0;
+#pragma unroll 1
+        for (int j = 0; j < kPairs; ++j)
+            inside += disc_pair(e);
+    }
+    return inside;
+}
+
+// The sums run in chunks with a 32-bit counter and an unroll of 32: loop
+// bookkeeping then costs little beside the step (the MWC sum measured 11 %
+// faster on GB300 than with a 64-bit counter and an unroll of 8; the other
+// kinds were unchanged).  256 values of 24 bits fit 32: their chunks add up
+// in 32 bits, one shifted add per output in place of a shift and a 64-bit
+// add.
 template <int OP, int KIND>
 __device__ __forceinline__ uint64_t consume(Engine<KIND> &e, uint64_t m)
 {
     uint64_t acc = 0;
-    if constexpr (OP == RNG_SUM_U32 || OP == RNG_SUM_U24) {
+    if constexpr (OP == RNG_SUM_U32) {
         for (uint64_t done = 0; done < m;) {
             const uint32_t k = (uint32_t)(m - done < (1u << 30) ? m - done : (1u << 30));
 #pragma unroll 32
-            for (uint32_t j = 0; j < k; ++j) {
-                if constexpr (OP == RNG_SUM_U32)
-                    acc += e.next();
-                else
-                    acc += e.next() >> 8;
-            }
+            for (uint32_t j = 0; j < k; ++j)
+                acc += next_of(e);
             done += k;
         }
-    } else {
-        // pairs (u0, u1): inside when (u0>>8)^2 + (u1>>8)^2 < 2^48
-#pragma unroll 4
-        for (uint64_t j = 1; j < m; j += 2) {
-            const uint64_t X = e.next() >> 8;
-            const uint64_t Y = e.next() >> 8;
-            acc += (X * X + Y * Y) >> 48 == 0 ? 1u : 0u;
+    } else if constexpr (OP == RNG_SUM_U24) {
+        for (; m >= 256; m -= 256) {
+            uint32_t part = 0;
+#pragma unroll 32
+            for (int j = 0; j < 256; ++j)
+                part += next_of(e) >> 8;
+            acc += part;
         }
+        uint32_t part = 0;
+        for (uint32_t j = 0; j < (uint32_t)m; ++j)
+            part += next_of(e) >> 8;
+        acc += part;
+    } else {
+        // kPairs pairs at a time by disc_block, the rest one by one
+        uint64_t left = m / 2;
+        for (; left >= kPairs; left -= kPairs)
+            acc += disc_block(e);
+        for (; left; --left)
+            acc += disc_pair(e);
         if (m & 1)
-            e.next();  // the unpaired last output is drawn and ignored
+            next_of(e);  // the unpaired last output is drawn and ignored
     }
     return acc;
 }
