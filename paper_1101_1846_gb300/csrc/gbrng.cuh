@@ -91,17 +91,28 @@ int one_cta_smem(const void *kernel, int threads);
 int launch_generate(int kind, int fmt, const GenLaunch &p, cudaStream_t st);
 // generate_paper.cu: the same for RNG_MWC16X2, RNG_XORSHIFT8, RNG_KISS_XOR.
 int launch_generate_paper(int kind, int fmt, const GenLaunch &p, cudaStream_t st);
-// Segments of a split call: rows per segment (a power of two) and count
-// (at most max_segments); returns false when the call should run unsplit.
-// `streams` are the streams the call advances, `streams_per_thread` how many
-// of them one thread takes.
-// fill_threads: the threads the segments should add up to (split_fill).
-bool split_plan(int kind, uint64_t streams, uint64_t steps, uint64_t streams_per_thread,
-                uint64_t max_segments, uint64_t fill_threads, uint64_t *rows,
-                uint64_t *segments);
-// Threads a split call aims for: generate calls, or consumer
-// (rng_generate_reduce) calls.
-uint64_t split_fill(bool reduce);
+// CTAs of `threads` threads and `smem` bytes of dynamic shared memory of
+// `kernel` that the device holds at once (remembered); sets the kernel's
+// shared-memory limit.  0 when the device cannot tell.
+int resident_ctas(const void *kernel, int threads, int smem);
+
+// Whether a call that advances `streams` streams `steps` times is split into
+// segments.
+enum class SplitForm {
+    kAligned,  // generate, 16-byte rows: four streams per thread
+    kShifted,  // generate, other rows: four streams per thread
+    kReduce    // consumers: one stream per thread
+};
+bool split_wanted(int kind, SplitForm form, uint64_t streams, uint64_t steps);
+// Its segments, for `tiles` CTAs per segment and `resident` CTAs on the device
+// at once (0: unknown).  False when there would be only one.
+struct Segments {
+    uint64_t rows;   // per segment (even)
+    uint64_t count;  // at most max_segments
+    bool table;      // MWC32, KISS: worth the handle's table of powers
+};
+bool split_segments(int kind, SplitForm form, uint64_t streams, uint64_t steps, uint64_t tiles,
+                    uint64_t resident, uint64_t max_segments, Segments *out);
 
 // jump.cu: device tables of the GF(2) and affine jumps, built on first use
 // on the current device (synchronises then).

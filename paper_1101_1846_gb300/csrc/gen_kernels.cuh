@@ -92,14 +92,24 @@ gen_shift(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult, uint6
                                 (uint32_t)(left < per_cta ? left : per_cta));
 }
 
-// Warps of groups per CTA of gen_split_shift (249 groups), beside its tail warp.
-constexpr int kShiftSplitWarps = 8;
+// Dynamic shared memory (nothing is stored there) that keeps gen_split of 16-
+// but not 32-byte rows to three CTAs of 256 threads per SM: as in the
+// barrier-synced kernels, fewer warps writing at once keep the write stream
+// denser.  76,636 x 4096 on GB300, us a call without it and with it: MWC 221
+// -> 189, KISS 209 -> 191, MWC16X2 194 -> 189 (two per SM: 397, 378 and 395 at
+// 8192 rows, against 377, 382 and 379 with three and 447, 415 and 417 without);
+// KISS_XOR, bound by its arithmetic, keeps as many as fit.
+constexpr int kSyncSplitSmem = 60 * 1024;
+
+// Warps of groups per CTA of gen_split_shift (125 groups), beside its tail warp.
+constexpr int kShiftSplitWarps = 4;
 
 // Sequence splitting (Sec. "Parallelizing RNGs") for calls with too few
 // streams to fill the device: segment y of the grid produces rows
 // [y*rows, min(steps, (y+1)*rows)) of every stream, starting from the state
 // jumped ahead by y*rows steps (the MWC part by the handle's tabulated
-// multiplier a^(y*rows), the xorshift and LCG parts by the device tables).
+// multiplier a^(y*rows), the xorshift and LCG parts, which all streams of a
+// segment share, composed by each CTA from the device tables: SegmentJump).
 // One group of four streams per thread, rows 32-byte aligned (as gen_vec).
 //
 // Writing the final state back must wait until every segment has read the
@@ -124,8 +134,6 @@ gen_split(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult, uint6
 {
     uint64_t c_first = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
     const bool live = c_first < count;
-    if (!SYNC && !live)
-        return;
     if (!live)
         c_first = 0;  // compute on stream 0's state, never store
     constexpr int W = KindTraits<KIND>::W;
@@ -155,9 +163,10 @@ gen_split(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult, uint6
         *cnt = 0;
     }
     if (y > 0) {
+        __shared__ SegmentJump<KIND> jump;
+        jump.fill(first, T);
         // MWC32 / KISS: the tabulated a^(y*rows) when the handle's table is
         // passed, else powering (calls captured in a CUDA graph)
-        bool mwc_done = false;
         if constexpr (KIND == RNG_MWC32 || KIND == RNG_KISS) {
             if (jmul) {
                 const uint4 lo =
@@ -166,17 +175,17 @@ gen_split(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult, uint6
                     __ldg(reinterpret_cast<const uint4 *>(jmul + (uint64_t)y * n + s0 + 2));
                 const uint64_t A[4] = {(uint64_t)lo.y << 32 | lo.x, (uint64_t)lo.w << 32 | lo.z,
                                        (uint64_t)hi.y << 32 | hi.x, (uint64_t)hi.w << 32 | hi.z};
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    mwc_apply(A[i], a[i], w[0][i], w[1][i]);
-                mwc_done = true;
+                mwc_jump_streams<KIND, 4>(w, a, first, A);
+            } else {
+                mwc_jump_streams<KIND, 4>(w, a, first, nullptr);
             }
+        } else {
+            mwc_jump_streams<KIND, 4>(w, a, first, nullptr);
         }
-        if (mwc_done)
-            jump_streams<KIND, 4, true>(w, a, first, T);
-        else
-            jump_streams<KIND, 4, false>(w, a, first, T);
+        jump.template apply<4>(w);
     }
+    if (!SYNC && !live)
+        return;  // after the CTA's part of the jump
     uint32_t *row = out + (uint64_t)first * ld + c_first;
     if constexpr (SYNC) {
         for (uint32_t j = 0; j < mine; ++j) {
@@ -227,14 +236,35 @@ gen_split(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult, uint6
 // arrival, so the arrivals of owners and tail lanes (one counter per first
 // stream) cover every read.
 //
-// The row's alignment is uniform over the CTA and chosen at run time, in
-// blocks of four rows (so that xor128's words are renamed, not moved): a
-// compile-time sequence as in gen_shift would double the longest compile
-// and a split call is bound by its jumps, its launch or the write stream.
+// The row's alignment r is uniform over the CTA and goes through r, r + dr, ..
+// mod 4 (dr = ld mod 4), a cycle of at most four rows: up to three rows with r
+// chosen at run time lead to the cycle's fixed start (shift_cycle_start), the
+// blocks of four rows that follow have every r at compile time (eight
+// sequences, where gen_shift, which starts at any r, has sixteen, in two
+// forms), and at most three rows are left.
 // MWC powers are taken in the kernel when the handle's table does not already
 // hold them: this path never allocates and never waits.
-// Split against whole calls on GB300: KISS f32 1001 x 16384 1592 -> 47.9
-// us a call.
+// On GB300, us a call, whole calls -> this: KISS f32 1001 x 16384 1587 -> 30.7
+// (46.6 with a run-time alignment and 32 columns per set bit of the jump), KISS
+// u32 10,001 x 8192 370 -> 79, MWC 76,633 x 4096 278 -> 194.
+template <int KIND, int FMT, int HINT, int R0, int DR>
+__device__ __forceinline__ void shift_cycle(uint32_t (&w)[kMaxWords][4], const uint32_t (&a)[4],
+                                            uint32_t *&row, uint64_t ld, uint32_t blocks,
+                                            bool owner, bool prev, bool next, bool lead,
+                                            bool trail)
+{
+    OutMap m;
+    shift_rows<KIND, FMT, HINT, R0, DR, true>(w, a, row, ld, blocks, owner, prev, next, lead,
+                                              trail, m);
+}
+
+// Rows until the alignment is one that shift_cycle has: 0 for dr = 1 and 3
+// (the cycle has all four), 0 or 1 for dr = 2, any for dr = 0.
+__device__ __forceinline__ uint32_t shift_cycle_start(uint32_t r, uint32_t dr)
+{
+    return dr == 0 ? 0 : dr == 1 ? (4 - r) & 3 : dr == 2 ? r >> 1 : r;
+}
+
 template <int KIND, int FMT, int HINT>
 __global__ void __launch_bounds__(32 * (kShiftSplitWarps + 1))
 gen_split_shift(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult, uint64_t n,
@@ -296,45 +326,74 @@ gen_split_shift(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult,
             *cnt = 0;
         }
     }
-    if (y > 0 && live) {
-        bool mwc_done = false;
-        if constexpr (KIND == RNG_MWC32 || KIND == RNG_KISS) {
-            if (jmul) {
+    if (y > 0) {
+        __shared__ SegmentJump<KIND> jump;
+        jump.fill(first, T);
+        if (live) {
+            if ((KIND == RNG_MWC32 || KIND == RNG_KISS) && jmul) {
+                uint64_t A[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
-                    mwc_apply(__ldg(jmul + (uint64_t)y * n + s0 + (tail_warp ? 0 : i)), a[i],
-                              w[0][i], w[1][i]);
-                mwc_done = true;
+                    A[i] = __ldg(jmul + (uint64_t)y * n + s0 + (tail_warp ? 0 : i));
+                mwc_jump_streams<KIND, 4>(w, a, first, A);
+            } else {
+                mwc_jump_streams<KIND, 4>(w, a, first, nullptr);
             }
+            jump.template apply<4>(w);
         }
-        if (mwc_done)
-            jump_streams<KIND, 4, true>(w, a, first, T);
-        else
-            jump_streams<KIND, 4, false>(w, a, first, T);
     }
     uint32_t *row = out + (uint64_t)first * ld + c;
     if (!tail_warp && !live)
         row = out;  // never stored to; keeps the alignment's arithmetic in range
     const uint32_t dr = (uint32_t)(ld & 3);
     uint32_t r = (uint32_t)(((uintptr_t)(out + (uint64_t)first * ld) >> 2) & 3);
-    OutMap m;
-    for (uint32_t j = 0; j < n_rows; j += 4) {
-        if (j % KindTraits<KIND>::SYNC_ROWS == 0)
-            __syncthreads();
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            if (j + q < n_rows) {
-                if (tail_warp) {
-                    const uint32_t o = step_enc<KIND, FMT>(w, a, 0);
-                    if (live)
-                        store4<HINT>(row, o);
-                } else {
-                    shift_row_rt<KIND, FMT, HINT>(w, a, row, r, owner, prev, next, lead, trail, m);
-                }
-            }
+    const uint32_t lead_in = min(shift_cycle_start(r, dr), n_rows);
+    const uint32_t blocks = (n_rows - lead_in) / 4, rest = (n_rows - lead_in) % 4;
+    if (tail_warp) {
+        auto step = [&] {
+            const uint32_t o = step_enc<KIND, FMT>(w, a, 0);
+            if (live)
+                store4<HINT>(row, o);
+            row += ld;
+        };
+        for (uint32_t j = 0; j < lead_in; ++j)
+            step();
+        for (uint32_t b = 0; b < blocks; ++b) {
+            if (b % (KindTraits<KIND>::SYNC_ROWS / 4) == 0)
+                __syncthreads();  // with shift_rows
+            step();
+            step();
+            step();
+            step();
+        }
+        for (uint32_t j = 0; j < rest; ++j)
+            step();
+    } else {
+        OutMap m;
+        auto one = [&] {
+            shift_row_rt<KIND, FMT, HINT>(w, a, row, r, owner, prev, next, lead, trail, m);
             row += ld;
             r = (r + dr) & 3u;
-        }
+        };
+#pragma unroll 1
+        for (uint32_t j = 0; j < lead_in; ++j)
+            one();
+#define GBRNG_SHIFT_CYCLE(R0_, DR_)                                                             \
+    case (DR_) * 4 + (R0_):                                                                     \
+        shift_cycle<KIND, FMT, HINT, R0_, DR_>(w, a, row, ld, blocks, owner, prev, next, lead,  \
+                                               trail);                                          \
+        break;
+        if (blocks)
+            switch (dr * 4 + r) {
+                GBRNG_SHIFT_CYCLE(0, 0) GBRNG_SHIFT_CYCLE(1, 0) GBRNG_SHIFT_CYCLE(2, 0)
+                GBRNG_SHIFT_CYCLE(3, 0) GBRNG_SHIFT_CYCLE(0, 1) GBRNG_SHIFT_CYCLE(0, 2)
+                GBRNG_SHIFT_CYCLE(1, 2) GBRNG_SHIFT_CYCLE(0, 3)
+            default: break;
+            }
+#undef GBRNG_SHIFT_CYCLE
+#pragma unroll 1
+        for (uint32_t j = 0; j < rest; ++j)
+            one();
     }
     if (y == segs - 1 && owner) {
         save(stash);
@@ -452,6 +511,94 @@ void pick_vec(int v, int hint,
     vec = hint ? gen_vec<KIND, FMT, 1, 1> : gen_vec<KIND, FMT, 1, 0>;
 }
 
+// Whether a call on `st` may use the handle's MWC table.  Inside a CUDA graph
+// capture it is not (re)built: its kernel would only run at replay while later
+// direct calls took it as ready.  Nor does a captured call keep its address:
+// it may grow.
+inline int table_allowed(cudaStream_t st, bool *allowed)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const int e = cuda_status(cudaStreamIsCapturing(st, &cap));
+    *allowed = !e && cap == cudaStreamCaptureStatusNone;
+    return e;
+}
+
+// A split call with 16-byte rows.  *done: launched (else it would have had a
+// single segment).
+template <int KIND>
+int launch_split(int fmt, int hint, bool sectors, const GenLaunch &p, cudaStream_t st, bool *done)
+{
+    using Fn = void (*)(uint32_t *, const uint32_t *, uint64_t, uint32_t, uint32_t, uint32_t *,
+                        uint64_t, uint64_t, uint64_t, uint32_t *, uint32_t *, const uint64_t *,
+                        JumpTables);
+    Fn fn;
+    if (sectors)
+        fn = fmt == RNG_F32 ? (hint ? gen_split<KIND, RNG_F32, 1, false>
+                                    : gen_split<KIND, RNG_F32, 0, false>)
+                            : (hint ? gen_split<KIND, RNG_U32, 1, false>
+                                    : gen_split<KIND, RNG_U32, 0, false>);
+    else
+        fn = fmt == RNG_F32
+                 ? (hint ? gen_split<KIND, RNG_F32, 1, true> : gen_split<KIND, RNG_F32, 0, true>)
+                 : (hint ? gen_split<KIND, RNG_U32, 1, true> : gen_split<KIND, RNG_U32, 0, true>);
+    Gen *g = p.owner;
+    const uint64_t count = p.s_end - p.s_begin, tiles = (count / 4 + 255) / 256;
+    const int smem = !sectors && KIND != RNG_KISS_XOR ? kSyncSplitSmem : 0;
+    Segments seg;
+    if (!split_segments(KIND, SplitForm::kAligned, count, p.steps, tiles,
+                        resident_ctas((const void *)fn, 256, smem), g->jmul_segs, &seg))
+        return RNG_OK;
+    JumpTables T{};
+    const uint64_t *jmul = nullptr;
+    bool table = false;
+    int e = needs_jump_tables(KIND) ? jump_tables(&T) : RNG_OK;
+    if (!e && mont_table(KIND) && seg.table)
+        e = table_allowed(st, &table);
+    if (!e && table)
+        e = mwc_jump_table(g, seg.rows, seg.count, st, &jmul);
+    if (e)
+        return e;
+    *done = true;
+    fn<<<dim3((unsigned)tiles, (unsigned)seg.count), 256, smem, st>>>(
+        p.state, p.a, p.n, (uint32_t)p.steps, (uint32_t)seg.rows, static_cast<uint32_t *>(p.out),
+        p.ld, p.s_begin, count, g->d_split, g->d_cnt, jmul, T);
+    return cuda_status(cudaGetLastError());
+}
+
+// The same for rows that are not 16-byte aligned; never allocates or waits.
+template <int KIND>
+int launch_split_shift(int fmt, const GenLaunch &p, cudaStream_t st, bool *done)
+{
+    auto fn =
+        fmt == RNG_F32 ? gen_split_shift<KIND, RNG_F32, 1> : gen_split_shift<KIND, RNG_U32, 1>;
+    Gen *g = p.owner;
+    // groups spread evenly over as few CTAs per segment as hold them
+    const uint64_t count = p.s_end - p.s_begin;
+    const uint64_t groups = count / 4, most = 31 * kShiftSplitWarps + 1;
+    const uint64_t few = std::max<uint64_t>((groups + most - 1) / most, 1);
+    const uint64_t per = (groups + few - 1) / few;
+    const int warps = per < 2 ? (int)per : (int)((per - 1 + 30) / 31);
+    const uint64_t tiles = warps ? (groups + 31 * warps) / (31 * warps + 1) : 1;
+    const int threads = 32 * (warps + (count % 4 ? 1 : 0));
+    Segments seg;
+    if (!split_segments(KIND, SplitForm::kShifted, count, p.steps, tiles,
+                        resident_ctas((const void *)fn, threads, 0), g->jmul_segs, &seg))
+        return RNG_OK;
+    JumpTables T{};
+    bool table = false;
+    int e = needs_jump_tables(KIND) ? jump_tables(&T) : RNG_OK;
+    if (!e && mont_table(KIND))
+        e = table_allowed(st, &table);
+    if (e)
+        return e;
+    *done = true;
+    fn<<<dim3((unsigned)tiles, (unsigned)seg.count), threads, 0, st>>>(
+        p.state, p.a, p.n, (uint32_t)p.steps, (uint32_t)seg.rows, static_cast<uint32_t *>(p.out),
+        p.ld, p.s_begin, count, warps, g->d_split, g->d_cnt,
+        table ? ready_jump_table(g, seg.rows, seg.count) : nullptr, T);
+    return cuda_status(cudaGetLastError());
+}
+
 // One generate call of a KIND generator: picks the path from how the rows
 // sit in memory (aligned / synced / realigned), or splits a few-stream call
 // into jumped segments.
@@ -484,66 +631,14 @@ int launch_kind(int fmt, const GenLaunch &p, cudaStream_t st)
     const bool sectors = aligned && (p.ld % 8 == 0) && ((uintptr_t)p.out % 32 == 0);
     const uint64_t main = count & ~(uint64_t)3;
     uint32_t *out = static_cast<uint32_t *>(p.out);
-    uint64_t L = 0, S = 0;
     Gen *g = p.owner;
-    const bool split = g && g->d_split &&
-                       split_plan(KIND, count, p.steps, 4, g->jmul_segs, split_fill(false), &L, &S);
-    if (split && !aligned) {
-        JumpTables T{};
-        int e = needs_jump_tables(KIND) ? jump_tables(&T) : RNG_OK;
-        // a captured call must not keep the table's address: it may grow later
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (!e)
-            e = cuda_status(cudaStreamIsCapturing(st, &cap));
-        if (e)
+    const SplitForm form = aligned ? SplitForm::kAligned : SplitForm::kShifted;
+    if (g && g->d_split && split_wanted(KIND, form, count, p.steps)) {
+        bool done = false;
+        const int e = aligned ? launch_split<KIND>(fmt, sh.hint, sectors, p, st, &done)
+                              : launch_split_shift<KIND>(fmt, p, st, &done);
+        if (e || done)
             return e;
-        const uint64_t *jmul =
-            cap == cudaStreamCaptureStatusNone ? ready_jump_table(g, L, S) : nullptr;
-        // groups spread evenly over as few CTAs per segment as hold them
-        const uint64_t groups = main / 4, most = 31 * kShiftSplitWarps + 1;
-        const uint64_t few = std::max<uint64_t>((groups + most - 1) / most, 1);
-        const uint64_t per = (groups + few - 1) / few;
-        const int warps = per < 2 ? (int)per : (int)((per - 1 + 30) / 31);
-        const uint64_t tiles = warps ? (groups + 31 * warps) / (31 * warps + 1) : 1;
-        const int threads = 32 * (warps + (count > main ? 1 : 0));
-        auto fn = fmt == RNG_F32 ? gen_split_shift<KIND, RNG_F32, 1>
-                                 : gen_split_shift<KIND, RNG_U32, 1>;
-        fn<<<dim3((unsigned)tiles, (unsigned)S), threads, 0, st>>>(
-            p.state, p.a, p.n, (uint32_t)p.steps, (uint32_t)L, out, p.ld, p.s_begin, count, warps,
-            g->d_split, g->d_cnt, jmul, T);
-        return cuda_status(cudaGetLastError());
-    }
-    if (split) {
-        JumpTables T{};
-        const uint64_t *jmul = nullptr;
-        int e = needs_jump_tables(KIND) ? jump_tables(&T) : RNG_OK;
-        // Inside a CUDA graph capture the table is not (re)built: its kernel
-        // would only run at replay while later direct calls took it as ready.
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (!e)
-            e = cuda_status(cudaStreamIsCapturing(st, &cap));
-        if (!e && mont_table(KIND) && cap == cudaStreamCaptureStatusNone)
-            e = mwc_jump_table(g, L, S, st, &jmul);
-        if (e)
-            return e;
-        using SplitFn = void (*)(uint32_t *, const uint32_t *, uint64_t, uint32_t, uint32_t,
-                                 uint32_t *, uint64_t, uint64_t, uint64_t, uint32_t *,
-                                 uint32_t *, const uint64_t *, JumpTables);
-        SplitFn fn;
-        if (sectors)
-            fn = fmt == RNG_F32 ? (sh.hint ? gen_split<KIND, RNG_F32, 1, false>
-                                           : gen_split<KIND, RNG_F32, 0, false>)
-                                : (sh.hint ? gen_split<KIND, RNG_U32, 1, false>
-                                           : gen_split<KIND, RNG_U32, 0, false>);
-        else
-            fn = fmt == RNG_F32 ? (sh.hint ? gen_split<KIND, RNG_F32, 1, true>
-                                           : gen_split<KIND, RNG_F32, 0, true>)
-                                : (sh.hint ? gen_split<KIND, RNG_U32, 1, true>
-                                           : gen_split<KIND, RNG_U32, 0, true>);
-        const dim3 grid((unsigned)((count / 4 + 255) / 256), (unsigned)S);
-        fn<<<grid, 256, 0, st>>>(p.state, p.a, p.n, (uint32_t)p.steps, (uint32_t)L, out, p.ld,
-                                 p.s_begin, count, g->d_split, g->d_cnt, jmul, T);
-        return cuda_status(cudaGetLastError());
     }
     // Calls longer than 2^31 steps are cut into pieces (the kernels count
     // steps in 32 bits); the state carries from piece to piece.

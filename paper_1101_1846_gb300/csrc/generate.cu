@@ -83,22 +83,78 @@ int g_row_ctas[kKinds][2][2] = {
     {{0, 0}, {0, 0}},  // KISS_XOR
 };
 
-// Fewest rows of a split segment, as log2, per kind (0: never split).  The
-// jump that starts a segment costs about as much as this many rows: MWC32 a
-// tabulated Montgomery product, KISS that plus 32-column GF(2) products,
-// xor128 128-column products, the base-2^16 MWC parts a 32-bit Montgomery
-// powering each; XORSHIFT8's 256-column products cost more than splitting
-// gains.
-int g_split_log2[kKinds] = {6, 8, 7, 8, 0, 8};
+// Fewest rows of a split segment, as log2, per kind (0: never split), and
+// the rows it has when that gives threads enough.  The jump that starts a
+// segment costs about as much as the fewest rows: MWC32 a Montgomery product
+// or a power, the base-2^16 parts a 32-bit power each, the KISS kinds that and
+// the CTA's composed maps, xor128 and XORSHIFT8 a composed matrix (SegmentJump).
+// A call that has all the threads it wants takes segments of equal length,
+// any multiple of eight rows (76,636 x 2400 MWC: 113 us with 16 of 152 rows, 121
+// with ten of 256), but for xor128 and XORSHIFT8, whose jumps compose a matrix
+// per set bit of the segment's first row (xor128 there: 124 us with 256 rows,
+// 145 with 200), and the consumers.  Its MWC powers are taken in the kernel:
+// against rows that long they cost nothing (76,632 x 4096: MWC 184 us with the
+// handle's table, 181 without; KISS 198 and 192), and calls of many lengths
+// rebuild no table.  Shorter segments keep powers of two and the table (MWC
+// 4096 x 4096: 15.0 us with it, 18.9 without).
+// From a sweep on GB300 of 32 ... 300,001 streams by 150 ... 16384 rows, every
+// kind, aligned and not, segments of 2^5 ... 2^11 rows and whole calls.
+int g_split_log2[kKinds] = {5, 7, 5, 5, 8, 5};
+constexpr int kSplitRowsLog2[kKinds] = {6, 8, 7, 7, 9, 8};
+// Consumer calls, one stream per thread, pay the same jumps for a quarter of
+// the work a row (XORSHIFT8 sums, whole -> split, us: 1000 x 8192 212 -> 60,
+// 10,000 x 8192 213 -> 132; 1000 x 65,536 1671 -> 125).
+constexpr int kReduceRowsLog2[kKinds] = {6, 8, 7, 8, 10, 8};
+// Fewer threads than this in all, and fewer CTAs than SMs: shorter segments,
+// down to the fewest rows.
+// (4099 x 1024 KISS: 16.5 us with 64 rows, 20.6 with 128; 1001 x 16384, which
+// reaches 32,000 threads with 128: 29.1 with 128, 32.0 with 64; 4096 x 4800
+// KISS_XOR: 22.7 with 128, 33.3 with 256, which has 19,000 threads.)
+constexpr uint64_t kSplitThreads[kKinds] = {16000, 16000, 16000, 16000, 16000, 40000};
+// No table for calls this short: their exponents are as short.
+constexpr uint64_t kNoTableSteps = 128;
 // Calls of fewer threads than half of this are "few-stream" calls, which
-// split when their rows allow.
+// split.
 constexpr uint64_t kFewStreamThreads = (uint64_t)kSMs * 1024;
-// Threads a split generate call aims for: 2048 per SM, the most that can be
+// Threads a split generate call may have: 2048 per SM, the most that can be
 // resident.  Against 1024 per SM this was measured on GB300 at
 // 76,632 x 16,384: MWC32 1584 -> 1740 GS/s, KISS 1575 -> 1680, xor128
 // 1575 -> 1670; at 76,636 x 16,384, MWC16X2 1449 -> 1500 and KISS_XOR
 // 1541 -> 1680.  Consumer (reduce) calls, one stream per thread, keep 1024.
 constexpr uint64_t kSplitFillThreads = (uint64_t)kSMs * 2048;
+
+// KISS_XOR, whose steps cost most of those with cheap jumps, runs best as one
+// wave of CTAs while its segments stay this short (76,636 x 4096 u32: 195 us in
+// one wave of 512-row segments, 204 in two; 40,004 x 4096 116 and 130; with
+// 1500 rows 590 in one, 545 in more).
+constexpr uint64_t kOneWaveRows = 512;
+
+inline uint64_t round8(uint64_t rows) { return (rows + 7) / 8 * 8; }
+
+inline uint64_t split_threads(SplitForm form, uint64_t streams)
+{
+    return form == SplitForm::kReduce ? streams : (streams + 3) / 4;
+}
+
+// Fewest rows of a call of `threads` threads a segment that is worth
+// splitting.  More threads fill more of the device as they are, and the jumps
+// of more segments cost more in all.  (xor128 40,001 x 1000: whole 38, split 50
+// us; 10,001 x 8192: 243 and 86.  XORSHIFT8 54,014 x 5838: whole 362, split
+// 431; 10,001 x 8192: 643 and 200.  KISS 150,001 x 300: whole 29, split 44;
+// 1001 x 300: 17.6 and 13.4.)
+uint64_t split_min_steps(int kind, SplitForm form, uint64_t threads)
+{
+    switch (kind) {
+    case RNG_XOR128: return std::max<uint64_t>(1024, std::min<uint64_t>(2048, threads * 3 / 10));
+    case RNG_XORSHIFT8: return std::max<uint64_t>(1024, threads * 3 / 5);
+    default: break;
+    }
+    if (kind == RNG_KISS_XOR)  // the slowest steps: the whole call takes longest
+        return form == SplitForm::kShifted ? threads / 50 : 0;
+    if (form == SplitForm::kShifted)
+        return std::max<uint64_t>(256, std::min<uint64_t>(1024, threads / 10));
+    return kind == RNG_MWC16X2 ? threads / 50 : 0;
+}
 
 }  // namespace
 
@@ -164,38 +220,81 @@ int one_cta_smem(const void *kernel, int threads)
     return smem;
 }
 
-uint64_t split_fill(bool reduce)
+int resident_ctas(const void *kernel, int threads, int smem)
 {
-    return reduce ? kFewStreamThreads : kSplitFillThreads;
+    struct Known {
+        const void *kernel;
+        int threads, smem, dev, ctas;
+    };
+    static std::mutex mu;
+    static std::vector<Known> known;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess)
+        return 0;
+    std::lock_guard<std::mutex> lock(mu);
+    for (const Known &k : known)
+        if (k.kernel == kernel && k.threads == threads && k.smem == smem && k.dev == dev)
+            return k.ctas;
+    int sms = 0, fit = 0;
+    if ((smem && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      smem) != cudaSuccess) ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kernel, threads, smem) !=
+            cudaSuccess) {
+        cudaGetLastError();  // leave no sticky error from the probe behind
+        fit = 0;
+    }
+    known.push_back(Known{kernel, threads, smem, dev, sms * fit});
+    return sms * fit;
 }
 
 uint32_t split_max_segments(uint64_t n)
 {
     const uint64_t threads = (n + 3) / 4;
-    const uint64_t fill = std::max(split_fill(false), split_fill(true));
-    return (uint32_t)std::min<uint64_t>(fill / std::max<uint64_t>(threads, 1), 65535);
+    return (uint32_t)std::min<uint64_t>(kSplitFillThreads / std::max<uint64_t>(threads, 1), 65535);
 }
 
-bool split_plan(int kind, uint64_t streams, uint64_t steps, uint64_t streams_per_thread,
-                uint64_t max_segments, uint64_t fill_threads, uint64_t *rows,
-                uint64_t *segments)
+bool split_wanted(int kind, SplitForm form, uint64_t streams, uint64_t steps)
 {
-    const int l0 = g_split_log2[kind];
-    if (l0 == 0 || streams == 0 || streams > kSplitMaxStreams || steps > (1ull << 31))
+    if (g_split_log2[kind] == 0 || streams == 0 || streams > kSplitMaxStreams ||
+        steps > (1ull << 31))
         return false;
-    const uint64_t threads = (streams + streams_per_thread - 1) / streams_per_thread;
-    if (2 * threads > kFewStreamThreads)
-        return false;  // enough streams to fill the device already
-    const uint64_t want = std::min<uint64_t>(std::min<uint64_t>(fill_threads / threads, 65535),
-                                             max_segments);
-    uint64_t L = 1ull << l0;
-    while (L < steps && (steps + L - 1) / L > want)
+    const uint64_t threads = split_threads(form, streams);
+    return 2 * threads <= kFewStreamThreads &&  // else they fill the device already
+           steps >= split_min_steps(kind, form, threads);
+}
+
+bool split_segments(int kind, SplitForm form, uint64_t streams, uint64_t steps, uint64_t tiles,
+                    uint64_t resident, uint64_t max_segments, Segments *out)
+{
+    const bool reduce = form == SplitForm::kReduce;
+    const uint64_t threads = split_threads(form, streams);
+    const int fewest = g_split_log2[kind];
+    uint64_t want = std::min<uint64_t>(
+        std::min<uint64_t>((reduce ? kFewStreamThreads : kSplitFillThreads) / threads, 65535),
+        max_segments);
+    if (kind == RNG_KISS_XOR && !reduce && resident >= 2 * tiles &&
+        steps <= kOneWaveRows * (resident / tiles))
+        want = std::min(want, resident / tiles);
+    if (want < 2)
+        return false;
+    auto count = [&](uint64_t L) { return (steps + L - 1) / L; };
+    uint64_t L = 1ull << std::max(fewest, (reduce ? kReduceRowsLog2 : kSplitRowsLog2)[kind]);
+    while (!reduce && L > 1ull << fewest && threads * count(L) < kSplitThreads[kind] &&
+           tiles * count(L) < kSMs)
+        L >>= 1;
+    // as many segments as threads allow, each longer than L: of one length
+    const bool full = count(L) > want;
+    const bool gf2 = kind == RNG_XOR128 || kind == RNG_XORSHIFT8;
+    if (full && !reduce && !gf2) {
+        L = round8(count(want));
+        L = round8(count(count(L)));
+    }
+    while (L < steps && count(L) > want)
         L <<= 1;
-    const uint64_t S = (steps + L - 1) / L;
-    if (S < 2)
+    if (count(L) < 2)
         return false;
-    *rows = L;
-    *segments = S;
+    *out = Segments{L, count(L), reduce || (!full && steps > kNoTableSteps)};
     return true;
 }
 

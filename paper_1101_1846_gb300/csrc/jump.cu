@@ -161,15 +161,22 @@ __global__ void __launch_bounds__(256) jump_kernel(rng_device_view v, uint64_t k
         return;
     Engine<KIND> e;
     e.load(v, s);
-    if (!compose) {
-        jump_engine<KIND>(e, k, T);
-    } else if constexpr (KIND == RNG_KISS) {
+    if constexpr (KIND == RNG_MWC32 || KIND == RNG_KISS) {
         mwc_jump(e.a, e.x, e.c, k);
-        kiss_jump_apply(J, e.y, e.z);
-    } else if constexpr (KIND == RNG_KISS_XOR) {
+    } else {
         mwc16_jump(e.a & 0xFFFFu, e.z, k);
         mwc16_jump(e.a >> 16, e.w, k);
-        kiss_jump_apply(J, e.y, e.l);
+    }
+    if constexpr (KIND == RNG_KISS) {
+        if (compose)
+            kiss_jump_apply(J, e.y, e.z);
+        else
+            kiss_jump_bits(e.y, e.z, k, T);
+    } else if constexpr (KIND == RNG_KISS_XOR) {
+        if (compose)
+            kiss_jump_apply(J, e.y, e.l);
+        else
+            kiss_jump_bits(e.y, e.l, k, T);
     }
     e.store(v, s);
 }

@@ -104,79 +104,6 @@ __device__ __forceinline__ void mwc16_jump(uint32_t a, uint32_t &z, uint64_t k)
     z = mont_mul32(A, z, p, ninv);  // a^k R z R^-1 mod p
 }
 
-// v <- M v for a 128 x 128 GF(2) matrix given by columns (word w of column j
-// in col[j]); the four streams of a group share every column load.
-template <int G>
-__device__ __forceinline__ void gf2_apply128(const uint4 *__restrict__ col,
-                                             uint32_t (&w)[kMaxWords][4])
-{
-    uint32_t r[4][G];
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
-        for (int i = 0; i < G; ++i)
-            r[q][i] = 0;
-#pragma unroll
-    for (int word = 0; word < 4; ++word) {
-#pragma unroll 4
-        for (int b = 0; b < 32; ++b) {
-            const uint4 m = __ldg(col + 32 * word + b);
-#pragma unroll
-            for (int i = 0; i < G; ++i) {
-                const uint32_t mask = 0u - ((w[word][i] >> b) & 1u);
-                r[0][i] ^= m.x & mask;
-                r[1][i] ^= m.y & mask;
-                r[2][i] ^= m.z & mask;
-                r[3][i] ^= m.w & mask;
-            }
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
-        for (int i = 0; i < G; ++i)
-            w[q][i] = r[q][i];
-}
-
-// v <- M v for a 256 x 256 GF(2) matrix: column j is col[2j] (words 0-3)
-// and col[2j + 1] (words 4-7).
-template <int G>
-__device__ __forceinline__ void gf2_apply256(const uint4 *__restrict__ col,
-                                             uint32_t (&w)[kMaxWords][4])
-{
-    uint32_t r[8][G];
-#pragma unroll
-    for (int q = 0; q < 8; ++q)
-#pragma unroll
-        for (int i = 0; i < G; ++i)
-            r[q][i] = 0;
-#pragma unroll
-    for (int word = 0; word < 8; ++word) {
-#pragma unroll 2
-        for (int b = 0; b < 32; ++b) {
-            const uint4 lo = __ldg(col + 2 * (32 * word + b));
-            const uint4 hi = __ldg(col + 2 * (32 * word + b) + 1);
-#pragma unroll
-            for (int i = 0; i < G; ++i) {
-                const uint32_t mask = 0u - ((w[word][i] >> b) & 1u);
-                r[0][i] ^= lo.x & mask;
-                r[1][i] ^= lo.y & mask;
-                r[2][i] ^= lo.z & mask;
-                r[3][i] ^= lo.w & mask;
-                r[4][i] ^= hi.x & mask;
-                r[5][i] ^= hi.y & mask;
-                r[6][i] ^= hi.z & mask;
-                r[7][i] ^= hi.w & mask;
-            }
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < 8; ++q)
-#pragma unroll
-        for (int i = 0; i < G; ++i)
-            w[q][i] = r[q][i];
-}
-
 __device__ __forceinline__ uint32_t gf2_apply32(const uint32_t *__restrict__ col, uint32_t y)
 {
     uint32_t r = 0;
@@ -301,124 +228,189 @@ __device__ __forceinline__ void kiss_jump_apply(const KissJump &J, uint32_t &y, 
     z = J.A * z + J.C;
 }
 
-// Jumps G streams held as w[word][i] (the vector bodies' layout; G = 1 for
-// a single stream) with multipliers a[i] by k steps.  With MWC_DONE the
-// base-2^32 MWC words are left alone (the caller has applied a tabulated
-// multiplier).
-template <int KIND, int G, bool MWC_DONE = false>
-__device__ __forceinline__ void jump_streams(uint32_t (&w)[kMaxWords][4],
-                                             const uint32_t (&a)[4], uint64_t k,
-                                             const JumpTables &T)
+// The same for one stream, a matrix per set bit of k.
+__device__ __forceinline__ void kiss_jump_bits(uint32_t &y, uint32_t &z, uint64_t k,
+                                               const JumpTables &T)
 {
-    if (k == 0)
-        return;
-    if constexpr ((KIND == RNG_MWC32 || KIND == RNG_KISS) && !MWC_DONE) {
-#pragma unroll
-        for (int i = 0; i < G; ++i)
-            mwc_jump(a[i], w[0][i], w[1][i], k);
-    }
-    if constexpr (KIND == RNG_MWC16X2 || KIND == RNG_KISS_XOR) {
-#pragma unroll
-        for (int i = 0; i < G; ++i) {
-            mwc16_jump(a[i] & 0xFFFFu, w[0][i], k);
-            mwc16_jump(a[i] >> 16, w[1][i], k);
-        }
-    }
-    if constexpr (KIND == RNG_XOR128) {
-        for (uint64_t r = k; r; r &= r - 1)
-            gf2_apply128<G>(T.xor128 + 128 * (__ffsll((long long)r) - 1), w);
-    }
-    if constexpr (KIND == RNG_XORSHIFT8) {
-        for (uint64_t r = k; r; r &= r - 1)
-            gf2_apply256<G>(T.xs8 + 512 * (__ffsll((long long)r) - 1), w);
-    }
-    if constexpr (KIND == RNG_KISS || KIND == RNG_KISS_XOR) {
-        for (uint64_t r = k; r; r &= r - 1) {
-            const int m = __ffsll((long long)r) - 1;
-            const uint2 lc = __ldg(T.lcg + m);
-#pragma unroll
-            for (int i = 0; i < G; ++i) {
-                w[2][i] = gf2_apply32(T.xs32 + 32 * m, w[2][i]);
-                w[3][i] = lc.x * w[3][i] + lc.y;
-            }
-        }
+    for (uint64_t r = k; r; r &= r - 1) {
+        const int m = __ffsll((long long)r) - 1;
+        const uint2 lc = __ldg(T.lcg + m);
+        y = gf2_apply32(T.xs32 + 32 * m, y);
+        z = lc.x * z + lc.y;
     }
 }
 
-// The same for one stream in an Engine.  A != 0 (MWC32, KISS): the MWC part
-// is multiplied by A = a^k in Montgomery form (a tabulated power) instead of
-// powering.
-template <int KIND>
-__device__ __forceinline__ void jump_engine(Engine<KIND> &e, uint64_t k, const JumpTables &T,
-                                            uint64_t A = 0)
+// The columns of M^k of a kind with a big GF(2) part, composed by the CTA from
+// the set bits' matrices, a few of which are in shared memory at a time.
+template <int W>
+struct __align__(16) Gf2Jump {
+    static constexpr int kAtOnce = W == 4 ? 4 : 2;
+    uint32_t level[kAtOnce][32 * W * W];
+    uint32_t col[32 * W * W];
+};
+
+// r <- M w for the G vectors of a thread (word q of vector i in w[q][i]; they
+// share every column read) and a matrix in shared memory.
+template <int W, int G, int N>
+__device__ __forceinline__ void gf2_apply(const uint32_t *col, uint32_t (&w)[N][G])
 {
-    uint32_t w[kMaxWords][4] = {};
-    uint32_t a[4] = {};
-    if constexpr (KIND == RNG_MWC32) {
-        w[0][0] = e.x;
-        w[1][0] = e.c;
-        a[0] = e.a;
-    } else if constexpr (KIND == RNG_XOR128) {
-        w[0][0] = e.s0;
-        w[1][0] = e.s1;
-        w[2][0] = e.s2;
-        w[3][0] = e.s3;
-    } else if constexpr (KIND == RNG_KISS) {
-        w[0][0] = e.x;
-        w[1][0] = e.c;
-        w[2][0] = e.y;
-        w[3][0] = e.z;
-        a[0] = e.a;
-    } else if constexpr (KIND == RNG_MWC16X2) {
-        w[0][0] = e.z;
-        w[1][0] = e.w;
-        a[0] = e.a;
-    } else if constexpr (KIND == RNG_XORSHIFT8) {
+    uint32_t r[W][G] = {};
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-            w[q][0] = e.v[q];
-    } else {
-        w[0][0] = e.z;
-        w[1][0] = e.w;
-        w[2][0] = e.y;
-        w[3][0] = e.l;
-        a[0] = e.a;
-    }
-    if constexpr (KIND == RNG_MWC32 || KIND == RNG_KISS) {
-        if (A != 0 && k != 0) {
-            mwc_apply(A, a[0], w[0][0], w[1][0]);
-            jump_streams<KIND, 1, true>(w, a, k, T);
-        } else {
-            jump_streams<KIND, 1>(w, a, k, T);
+    for (int word = 0; word < W; ++word) {
+#pragma unroll 8
+        for (int b = 0; b < 32; ++b) {
+            const uint4 *c = reinterpret_cast<const uint4 *>(col + W * (32 * word + b));
+#pragma unroll
+            for (int h = 0; h < W / 4; ++h) {
+                const uint4 m = c[h];
+#pragma unroll
+                for (int i = 0; i < G; ++i) {
+                    const uint32_t mask = 0u - ((w[word][i] >> b) & 1u);
+                    r[4 * h][i] ^= m.x & mask;
+                    r[4 * h + 1][i] ^= m.y & mask;
+                    r[4 * h + 2][i] ^= m.z & mask;
+                    r[4 * h + 3][i] ^= m.w & mask;
+                }
+            }
         }
-    } else {
-        jump_streams<KIND, 1>(w, a, k, T);
     }
-    if constexpr (KIND == RNG_MWC32) {
-        e.x = w[0][0];
-        e.c = w[1][0];
-    } else if constexpr (KIND == RNG_XOR128) {
-        e.s0 = w[0][0];
-        e.s1 = w[1][0];
-        e.s2 = w[2][0];
-        e.s3 = w[3][0];
-    } else if constexpr (KIND == RNG_KISS) {
-        e.x = w[0][0];
-        e.c = w[1][0];
-        e.y = w[2][0];
-        e.z = w[3][0];
-    } else if constexpr (KIND == RNG_MWC16X2) {
-        e.z = w[0][0];
-        e.w = w[1][0];
-    } else if constexpr (KIND == RNG_XORSHIFT8) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-            e.v[q] = w[q][0];
-    } else {
-        e.z = w[0][0];
-        e.w = w[1][0];
-        e.y = w[2][0];
-        e.l = w[3][0];
+    for (int q = 0; q < W; ++q)
+#pragma unroll
+        for (int i = 0; i < G; ++i)
+            w[q][i] = r[q][i];
+}
+
+// Fills J for k >= 1; every thread of the CTA (a multiple of 32) calls this.
+// A thread takes a column at a time through the levels in shared memory.
+template <int W>
+__device__ __forceinline__ void gf2_jump_fill(Gf2Jump<W> &J, uint64_t k,
+                                              const uint32_t *__restrict__ table)
+{
+    constexpr int kWords = 32 * W * W;
+    for (int i = threadIdx.x; i < kWords; i += blockDim.x)  // the identity
+        J.col[i] = (i % W) == (i / W) / 32 ? 1u << (i / W % 32) : 0u;
+    for (uint64_t r = k; r;) {
+        int levels = 0;
+        for (; levels < Gf2Jump<W>::kAtOnce && r; ++levels, r &= r - 1) {
+            const uint32_t *src = table + (size_t)kWords * (__ffsll((long long)r) - 1);
+            for (int i = 4 * threadIdx.x; i < kWords; i += 4 * blockDim.x)
+                copy16_async(&J.level[levels][i], src + i);
+        }
+        copies_done();
+#pragma unroll 1
+        for (int j = threadIdx.x; j < 32 * W; j += blockDim.x) {
+            uint32_t v[W][1];
+#pragma unroll
+            for (int q = 0; q < W; ++q)
+                v[q][0] = J.col[W * j + q];
+#pragma unroll 1
+            for (int m = 0; m < levels; ++m)
+                gf2_apply<W, 1, W>(J.level[m], v);
+#pragma unroll
+            for (int q = 0; q < W; ++q)
+                J.col[W * j + q] = v[q][0];
+        }
+        __syncthreads();
+    }
+}
+
+// w <- M w for the first G of a thread's four streams.
+template <int W, int G>
+__device__ __forceinline__ void gf2_jump_apply(const Gf2Jump<W> &J, uint32_t (&w)[kMaxWords][4])
+{
+    uint32_t v[W][G];
+#pragma unroll
+    for (int q = 0; q < W; ++q)
+#pragma unroll
+        for (int i = 0; i < G; ++i)
+            v[q][i] = w[q][i];
+    gf2_apply<W, G, W>(J.col, v);
+#pragma unroll
+    for (int q = 0; q < W; ++q)
+#pragma unroll
+        for (int i = 0; i < G; ++i)
+            w[q][i] = v[q][i];
+}
+
+// The part of a segment's jump that all its streams share, composed once per
+// CTA: a call's segments jump by first = y * rows, which has several set bits,
+// and each cost every stream a matrix before.
+template <int KIND>
+struct SegmentJump {
+    __device__ __forceinline__ void fill(uint64_t, const JumpTables &) {}
+    template <int G>
+    __device__ __forceinline__ void apply(uint32_t (&)[kMaxWords][4]) const
+    {
+    }
+};
+struct KissSegmentJump {
+    KissJump J;
+    __device__ __forceinline__ void fill(uint64_t k, const JumpTables &T)
+    {
+        kiss_jump_fill(J, k, T);
+    }
+    template <int G>
+    __device__ __forceinline__ void apply(uint32_t (&w)[kMaxWords][4]) const
+    {
+#pragma unroll
+        for (int i = 0; i < G; ++i)
+            kiss_jump_apply(J, w[2][i], w[3][i]);
+    }
+};
+template <>
+struct SegmentJump<RNG_KISS> : KissSegmentJump {
+};
+template <>
+struct SegmentJump<RNG_KISS_XOR> : KissSegmentJump {
+};
+template <>
+struct SegmentJump<RNG_XOR128> {
+    Gf2Jump<4> J;
+    __device__ __forceinline__ void fill(uint64_t k, const JumpTables &T)
+    {
+        gf2_jump_fill<4>(J, k, reinterpret_cast<const uint32_t *>(T.xor128));
+    }
+    template <int G>
+    __device__ __forceinline__ void apply(uint32_t (&w)[kMaxWords][4]) const
+    {
+        gf2_jump_apply<4, G>(J, w);
+    }
+};
+template <>
+struct SegmentJump<RNG_XORSHIFT8> {
+    Gf2Jump<8> J;
+    __device__ __forceinline__ void fill(uint64_t k, const JumpTables &T)
+    {
+        gf2_jump_fill<8>(J, k, reinterpret_cast<const uint32_t *>(T.xs8));
+    }
+    template <int G>
+    __device__ __forceinline__ void apply(uint32_t (&w)[kMaxWords][4]) const
+    {
+        gf2_jump_apply<8, G>(J, w);
+    }
+};
+
+// Jumps the MWC parts of G streams held as w[word][i] (the vector bodies'
+// layout) with multipliers a[i] by k steps; A (MWC32, KISS): the tabulated
+// powers a[i]^k in Montgomery form, or nullptr.
+template <int KIND, int G>
+__device__ __forceinline__ void mwc_jump_streams(uint32_t (&w)[kMaxWords][4],
+                                                 const uint32_t (&a)[4], uint64_t k,
+                                                 const uint64_t *A)
+{
+#pragma unroll
+    for (int i = 0; i < G; ++i) {
+        if constexpr (KIND == RNG_MWC32 || KIND == RNG_KISS) {
+            if (A)
+                mwc_apply(A[i], a[i], w[0][i], w[1][i]);
+            else
+                mwc_jump(a[i], w[0][i], w[1][i], k);
+        }
+        if constexpr (KIND == RNG_MWC16X2 || KIND == RNG_KISS_XOR) {
+            mwc16_jump(a[i] & 0xFFFFu, w[0][i], k);
+            mwc16_jump(a[i] >> 16, w[1][i], k);
+        }
     }
 }
 

@@ -23,10 +23,15 @@ constexpr int kThreads = 256;
 // that takes the adds off the FMA-heavy pipe, which bounds its consumers
 // (2^22 x 1024 on GB300: sum_u32 810 -> 699 us a call, disc 1029 -> 934), where
 // KISS, whose ALU pipe is as full, would lose 2-5 % by it.
-template <int KIND>
+// disc steps the base-2^16 kinds as the generate kernels do (mwc16x2_step_fma).
+template <int KIND, bool DISC = false>
 __device__ __forceinline__ uint32_t next_of(Engine<KIND> &e)
 {
-    if constexpr (KIND == RNG_MWC32) {
+    if constexpr (KIND == RNG_MWC16X2 && DISC) {
+        return mwc16x2_step_fma(e.a, e.z, e.w);
+    } else if constexpr (KIND == RNG_KISS_XOR && DISC) {
+        return (mwc16x2_step_fma(e.a, e.z, e.w) ^ lcg_step(e.l)) + xorshift32_step(e.y);
+    } else if constexpr (KIND == RNG_MWC32) {
         uint32_t lo, hi;
         asm("{\n\t.reg .u64 q;\n\t.reg .u32 l, h;\n\t"
             "mul.wide.u32 q, %2, %3;\n\t"
@@ -47,8 +52,8 @@ __device__ __forceinline__ uint32_t next_of(Engine<KIND> &e)
 template <int KIND>
 __device__ __forceinline__ uint32_t disc_pair(Engine<KIND> &e)
 {
-    const uint64_t X = next_of(e) >> 8;
-    const uint64_t Y = next_of(e) >> 8;
+    const uint64_t X = next_of<KIND, true>(e) >> 8;
+    const uint64_t Y = next_of<KIND, true>(e) >> 8;
     return (X * X + Y * Y) >> 48 == 0 ? 1u : 0u;
 }
 
@@ -74,8 +79,8 @@ __device__ __forceinline__ uint32_t disc_block(Engine<KIND> &e)
     float least = 0x1p64f;
 #pragma unroll
     for (int j = 0; j < kPairs; ++j) {
-        const float f0 = __uint2float_rn(next_of(e));
-        const float f1 = __uint2float_rn(next_of(e));
+        const float f0 = __uint2float_rn(next_of<KIND, true>(e));
+        const float f1 = __uint2float_rn(next_of<KIND, true>(e));
         const float d = __fmaf_rn(f0, f0, __fmaf_rn(f1, f1, -0x1p64f));
         inside += __float_as_uint(d) >> 31;
         least = fminf(least, fabsf(d));
@@ -133,6 +138,50 @@ __device__ __forceinline__ uint64_t consume(Engine<KIND> &e, uint64_t m)
     return acc;
 }
 
+// An engine's state as the vector bodies hold one stream (w[word][0], a[0]),
+// and back.
+template <int KIND>
+__device__ __forceinline__ void engine_words(const Engine<KIND> &e, uint32_t (&w)[kMaxWords][4],
+                                             uint32_t (&a)[4])
+{
+    if constexpr (KIND == RNG_MWC32) {
+        w[0][0] = e.x, w[1][0] = e.c, a[0] = e.a;
+    } else if constexpr (KIND == RNG_XOR128) {
+        w[0][0] = e.s0, w[1][0] = e.s1, w[2][0] = e.s2, w[3][0] = e.s3;
+    } else if constexpr (KIND == RNG_KISS) {
+        w[0][0] = e.x, w[1][0] = e.c, w[2][0] = e.y, w[3][0] = e.z, a[0] = e.a;
+    } else if constexpr (KIND == RNG_MWC16X2) {
+        w[0][0] = e.z, w[1][0] = e.w, a[0] = e.a;
+    } else if constexpr (KIND == RNG_XORSHIFT8) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            w[q][0] = e.v[q];
+    } else {
+        w[0][0] = e.z, w[1][0] = e.w, w[2][0] = e.y, w[3][0] = e.l, a[0] = e.a;
+    }
+}
+
+template <int KIND>
+__device__ __forceinline__ void engine_from_words(Engine<KIND> &e,
+                                                  const uint32_t (&w)[kMaxWords][4])
+{
+    if constexpr (KIND == RNG_MWC32) {
+        e.x = w[0][0], e.c = w[1][0];
+    } else if constexpr (KIND == RNG_XOR128) {
+        e.s0 = w[0][0], e.s1 = w[1][0], e.s2 = w[2][0], e.s3 = w[3][0];
+    } else if constexpr (KIND == RNG_KISS) {
+        e.x = w[0][0], e.c = w[1][0], e.y = w[2][0], e.z = w[3][0];
+    } else if constexpr (KIND == RNG_MWC16X2) {
+        e.z = w[0][0], e.w = w[1][0];
+    } else if constexpr (KIND == RNG_XORSHIFT8) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            e.v[q] = w[q][0];
+    } else {
+        e.z = w[0][0], e.w = w[1][0], e.y = w[2][0], e.l = w[3][0];
+    }
+}
+
 // SPLIT = false: one segment (grid y = 1), the whole call per thread.
 template <int KIND, int OP, bool SPLIT>
 __global__ void __launch_bounds__(kThreads)
@@ -141,33 +190,50 @@ reduce_kernel(rng_device_view v, uint64_t steps, uint64_t rows, uint64_t *__rest
               const uint64_t *__restrict__ jmul, JumpTables T)
 {
     const uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= v.n_streams)
-        return;
-    Engine<KIND> e;
-    e.load(v, s);
     if constexpr (!SPLIT) {
+        if (s >= v.n_streams)
+            return;
+        Engine<KIND> e;
+        e.load(v, s);
         out[s] = consume<OP>(e, steps);
         e.store(v, s);
         return;
     }
-    // Split: the same arrival count as gen_split (one counter per stream).
+    const bool live = s < v.n_streams;
     const uint32_t segs = gridDim.y;
     const uint64_t n = v.n_streams;
-    uint32_t *state = static_cast<uint32_t *>(v.state);
-    __threadfence();
-    uint32_t *cnt = counters + s;
-    if (atomicAdd(cnt, 1u) == segs) {
-        __threadfence();
-        for (int k = 0; k < v.state_words; ++k)
-            state[k * n + s] = __ldcg(stash + k * n + s);
-        *cnt = 0;
-    }
     const uint64_t first = (uint64_t)blockIdx.y * rows;
     const uint64_t mine = steps - first < rows ? steps - first : rows;
-    const uint64_t A = ((KIND == RNG_MWC32 || KIND == RNG_KISS) && blockIdx.y > 0 && jmul)
-                           ? jmul[blockIdx.y * n + s]
-                           : 0;
-    jump_engine<KIND>(e, first, T, A);
+    uint32_t *state = static_cast<uint32_t *>(v.state);
+    uint32_t *cnt = counters + s;
+    Engine<KIND> e;
+    // Split: the same arrival count as gen_split (one counter per stream).
+    if (live) {
+        e.load(v, s);
+        __threadfence();
+        if (atomicAdd(cnt, 1u) == segs) {
+            __threadfence();
+            for (int k = 0; k < v.state_words; ++k)
+                state[k * n + s] = __ldcg(stash + k * n + s);
+            *cnt = 0;
+        }
+    }
+    if (blockIdx.y > 0) {
+        __shared__ SegmentJump<KIND> jump;
+        jump.fill(first, T);
+        if (live) {
+            uint32_t w[kMaxWords][4] = {}, a[4] = {};
+            engine_words(e, w, a);
+            uint64_t A = 0;
+            if ((KIND == RNG_MWC32 || KIND == RNG_KISS) && jmul)
+                A = jmul[blockIdx.y * n + s];
+            mwc_jump_streams<KIND, 1>(w, a, first, A ? &A : nullptr);
+            jump.template apply<1>(w);
+            engine_from_words(e, w);
+        }
+    }
+    if (!live)
+        return;  // after the CTA's part of the jump
     atomicAdd(reinterpret_cast<unsigned long long *>(out + s),
               (unsigned long long)consume<OP>(e, mine));
     if (blockIdx.y == segs - 1) {
@@ -226,15 +292,13 @@ extern "C" int rng_generate_reduce(rng_handle h, uint64_t n_per_stream, int op, 
     cudaStream_t st = g->stream;
     uint64_t *o = static_cast<uint64_t *>(out);
     rng_device_view v{g->kind, g->device, g->words, g->n, g->d_state, g->d_a};
-    uint64_t rows = n_per_stream, segs = 1;
-    // pairs never straddle segments: split rows are powers of two >= 2
+    // pairs never straddle segments: their rows are an even number
+    Segments seg{n_per_stream, 1, false};
     const bool split = g->d_split &&
-                       split_plan(g->kind, g->n, n_per_stream, 1, g->jmul_segs,
-                                  split_fill(true), &rows, &segs);
-    if (!split) {
-        rows = n_per_stream;
-        segs = 1;
-    }
+                       split_wanted(g->kind, SplitForm::kReduce, g->n, n_per_stream) &&
+                       split_segments(g->kind, SplitForm::kReduce, g->n, n_per_stream,
+                                      (g->n + kThreads - 1) / kThreads, 0, g->jmul_segs, &seg);
+    const uint64_t rows = seg.rows, segs = seg.count;
     ReduceFn fn = split ? pick_kind<true>(g->kind, op) : pick_kind<false>(g->kind, op);
     JumpTables T{};
     const uint64_t *jmul = nullptr;
