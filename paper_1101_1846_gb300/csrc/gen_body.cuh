@@ -63,19 +63,20 @@ struct KindTraits<RNG_KISS_XOR> {
 // its first W, and the unused entries cost no registers.
 constexpr int kMaxWords = 8;
 
-// mwc16x2_step with the low halves and the joined output as multiply-adds: z
+// mwc16x2_step with work moved from the ALU pipe to the FMA pipe: the joined
+// output as a multiply-add, and the low halves of LOWS (0-2) of the parts, z
 // mod 2^16 = z - 2^16 (z div 2^16), written so that it is not turned back into
-// a mask.  The kinds built on it are bound by the ALU pipe where they are not
-// by the write stream (76,636 x 4096 KISS_XOR on GB300, segments of 512 rows,
-// us: u32 197 -> 194, f32 245 -> 216; its disc consumer 788 -> 763 at 16,384
-// rows; the sums, whose adds the compiler already moves, 682 -> 693, so they
-// keep mwc16x2_step).
+// a mask.  A part's recurrence is one instruction longer that way: for kernels
+// with enough warps.
+template <int LOWS>
 __device__ __forceinline__ uint32_t mwc16x2_step_fma(uint32_t a_pair, uint32_t &z, uint32_t &w)
 {
     const uint32_t hz = z >> 16, hw = w >> 16;
-    uint32_t lz, lw, out;
-    asm("mad.lo.u32 %0, %1, 0xFFFF0000, %2;" : "=r"(lz) : "r"(hz), "r"(z));
-    asm("mad.lo.u32 %0, %1, 0xFFFF0000, %2;" : "=r"(lw) : "r"(hw), "r"(w));
+    uint32_t lz = z & 0xFFFFu, lw = w & 0xFFFFu, out;
+    if constexpr (LOWS > 0)
+        asm("mad.lo.u32 %0, %1, 0xFFFF0000, %2;" : "=r"(lw) : "r"(hw), "r"(w));
+    if constexpr (LOWS > 1)
+        asm("mad.lo.u32 %0, %1, 0xFFFF0000, %2;" : "=r"(lz) : "r"(hz), "r"(z));
     z = (a_pair & 0xFFFFu) * lz + hz;
     w = (a_pair >> 16) * lw + hw;
     asm("mad.lo.u32 %0, %1, 0x10000, %2;" : "=r"(out) : "r"(z), "r"(w));
@@ -95,13 +96,12 @@ __device__ __forceinline__ uint32_t step_enc(uint32_t (&w)[kMaxWords][4],
     else if constexpr (KIND == RNG_KISS)
         u = kiss_step(a[i], w[0][i], w[1][i], w[2][i], w[3][i]);
     else if constexpr (KIND == RNG_MWC16X2)
-        u = mwc16x2_step_fma(a[i], w[0][i], w[1][i]);
+        u = mwc16x2_step(a[i], w[0][i], w[1][i]);
     else if constexpr (KIND == RNG_XORSHIFT8)
         u = xorshift8_step(w[0][i], w[1][i], w[2][i], w[3][i], w[4][i], w[5][i], w[6][i],
                            w[7][i]);
     else
-        u = (mwc16x2_step_fma(a[i], w[0][i], w[1][i]) ^ lcg_step(w[3][i])) +
-            xorshift32_step(w[2][i]);
+        u = kiss_xor_step(a[i], w[0][i], w[1][i], w[2][i], w[3][i]);
     if constexpr (FMT == RNG_F32)
         return __float_as_uint(unit_f32(u));
     else

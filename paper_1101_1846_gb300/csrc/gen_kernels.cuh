@@ -125,6 +125,23 @@ constexpr int kShiftSplitWarps = 4;
 // a shared DRAM sector meet in L2; every thread of the CTA then runs the
 // rows (a CTA shares its segment, hence its jump and its row count), and
 // threads past the last group store nothing and count no arrival.
+template <int KIND, int FMT>
+__device__ __forceinline__ uint32_t split_step(uint32_t (&w)[kMaxWords][4],
+                                               const uint32_t (&a)[4], int i)
+{
+    // KISS_XOR is bound by the ALU pipe here (76,636 x 4096, us: u32 194 with
+    // kiss_xor_step, 184 with the join alone moved, 192 with both low halves as
+    // well; f32, which adds a shift, a conversion and a product, 245, 230, 210)
+    if constexpr (KIND == RNG_KISS_XOR) {
+        const uint32_t u = (mwc16x2_step_fma<FMT == RNG_F32 ? 2 : 0>(a[i], w[0][i], w[1][i]) ^
+                            lcg_step(w[3][i])) +
+                           xorshift32_step(w[2][i]);
+        return FMT == RNG_F32 ? __float_as_uint(unit_f32(u)) : u;
+    } else {
+        return step_enc<KIND, FMT>(w, a, i);
+    }
+}
+
 template <int KIND, int FMT, int HINT, bool SYNC>
 __global__ void __launch_bounds__(256)
 gen_split(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult, uint64_t n,
@@ -191,10 +208,10 @@ gen_split(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult, uint6
         for (uint32_t j = 0; j < mine; ++j) {
             if (j % KindTraits<KIND>::SYNC_ROWS == 0)
                 __syncthreads();
-            const uint32_t o0 = step_enc<KIND, FMT>(w, a, 0);
-            const uint32_t o1 = step_enc<KIND, FMT>(w, a, 1);
-            const uint32_t o2 = step_enc<KIND, FMT>(w, a, 2);
-            const uint32_t o3 = step_enc<KIND, FMT>(w, a, 3);
+            const uint32_t o0 = split_step<KIND, FMT>(w, a, 0);
+            const uint32_t o1 = split_step<KIND, FMT>(w, a, 1);
+            const uint32_t o2 = split_step<KIND, FMT>(w, a, 2);
+            const uint32_t o3 = split_step<KIND, FMT>(w, a, 3);
             if (live)
                 store16<HINT>(row, o0, o1, o2, o3);
             row += ld;
@@ -204,10 +221,10 @@ gen_split(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult, uint6
     } else {
 #pragma unroll 4
         for (uint32_t j = 0; j < mine; ++j) {
-            const uint32_t o0 = step_enc<KIND, FMT>(w, a, 0);
-            const uint32_t o1 = step_enc<KIND, FMT>(w, a, 1);
-            const uint32_t o2 = step_enc<KIND, FMT>(w, a, 2);
-            const uint32_t o3 = step_enc<KIND, FMT>(w, a, 3);
+            const uint32_t o0 = split_step<KIND, FMT>(w, a, 0);
+            const uint32_t o1 = split_step<KIND, FMT>(w, a, 1);
+            const uint32_t o2 = split_step<KIND, FMT>(w, a, 2);
+            const uint32_t o3 = split_step<KIND, FMT>(w, a, 3);
             store16<HINT>(row, o0, o1, o2, o3);
             row += ld;
         }
@@ -482,6 +499,11 @@ gen_tma(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult, uint64_
 }
 
 constexpr int kSMs = 152;
+// 4096 x 128 u32 on GB300, device time of a whole call in us, two groups per
+// thread (MWC u32 by TMA: 8.6 for 4096 x 64) against one: MWC 8.7 and 5.4 (3.4),
+// KISS 12.9 and 7.3, xor128 9.8 and 4.8, MWC16X2 8.5 and 5.0, KISS_XOR 14.0 and
+// 7.6 (9.9 with streaming stores).
+constexpr uint64_t kSmallCall = (uint64_t)kSMs * 1024;
 // CTA size of the kernels with row barriers: large CTAs leave fewer CTA
 // boundaries, where neighbouring CTAs that drift apart split sectors.
 constexpr int kSyncBlock = 512;
@@ -610,7 +632,18 @@ int launch_kind(int fmt, const GenLaunch &p, cudaStream_t st)
     const uint64_t count = p.s_end - p.s_begin;
     if (p.steps == 0 || count == 0)
         return RNG_OK;
-    const LaunchShape sh = launch_shape(KIND, fmt, count);
+    LaunchShape sh = launch_shape(KIND, fmt, count);
+    const int split_hint = sh.hint;
+    // The shape is for calls that fill the device.  Below kSmallCall streams
+    // there is less than a CTA of it per SM: one group of four per thread then
+    // (two halve the warps), and 16-byte stores (TMA rows come in CTAs of 1024
+    // streams).  A single warp holds one group per thread anyway, and the
+    // fewest rows are over before it matters.
+    if (count < kSmallCall &&
+        (sh.hint == 2 || (sh.v == 2 && count > 128 && p.steps >= 16))) {
+        sh.v = 1;
+        sh.hint = 0;
+    }
     Fn vec, shift, sync;
     if (fmt == RNG_F32) {
         pick_vec<KIND, RNG_F32>(sh.v, sh.hint, vec);
@@ -635,7 +668,7 @@ int launch_kind(int fmt, const GenLaunch &p, cudaStream_t st)
     const SplitForm form = aligned ? SplitForm::kAligned : SplitForm::kShifted;
     if (g && g->d_split && split_wanted(KIND, form, count, p.steps)) {
         bool done = false;
-        const int e = aligned ? launch_split<KIND>(fmt, sh.hint, sectors, p, st, &done)
+        const int e = aligned ? launch_split<KIND>(fmt, split_hint, sectors, p, st, &done)
                               : launch_split_shift<KIND>(fmt, p, st, &done);
         if (e || done)
             return e;

@@ -149,11 +149,14 @@ uint64_t split_min_steps(int kind, SplitForm form, uint64_t threads)
     case RNG_XORSHIFT8: return std::max<uint64_t>(1024, threads * 3 / 5);
     default: break;
     }
+    // shorter calls take 4-8 us whole, one group per thread (kSmallCall), and as
+    // long split
+    const uint64_t least = 129;
     if (kind == RNG_KISS_XOR)  // the slowest steps: the whole call takes longest
-        return form == SplitForm::kShifted ? threads / 50 : 0;
+        return std::max(least, form == SplitForm::kShifted ? threads / 50 : 0);
     if (form == SplitForm::kShifted)
         return std::max<uint64_t>(256, std::min<uint64_t>(1024, threads / 10));
-    return kind == RNG_MWC16X2 ? threads / 50 : 0;
+    return std::max(least, kind == RNG_MWC16X2 ? threads / 50 : 0);
 }
 
 }  // namespace

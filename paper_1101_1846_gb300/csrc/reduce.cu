@@ -23,14 +23,17 @@ constexpr int kThreads = 256;
 // that takes the adds off the FMA-heavy pipe, which bounds its consumers
 // (2^22 x 1024 on GB300: sum_u32 810 -> 699 us a call, disc 1029 -> 934), where
 // KISS, whose ALU pipe is as full, would lose 2-5 % by it.
-// disc steps the base-2^16 kinds as the generate kernels do (mwc16x2_step_fma).
+// disc steps the base-2^16 kinds with one part's low half on the FMA pipe
+// (76,636 x 4096: MWC16X2 110 us without it, 103 with it, 106 with both parts';
+// KISS_XOR 202, 191 and 196; the sums are faster with mwc16x2_step, 682 against
+// 693 at 16,384 rows).
 template <int KIND, bool DISC = false>
 __device__ __forceinline__ uint32_t next_of(Engine<KIND> &e)
 {
     if constexpr (KIND == RNG_MWC16X2 && DISC) {
-        return mwc16x2_step_fma(e.a, e.z, e.w);
+        return mwc16x2_step_fma<1>(e.a, e.z, e.w);
     } else if constexpr (KIND == RNG_KISS_XOR && DISC) {
-        return (mwc16x2_step_fma(e.a, e.z, e.w) ^ lcg_step(e.l)) + xorshift32_step(e.y);
+        return (mwc16x2_step_fma<1>(e.a, e.z, e.w) ^ lcg_step(e.l)) + xorshift32_step(e.y);
     } else if constexpr (KIND == RNG_MWC32) {
         uint32_t lo, hi;
         asm("{\n\t.reg .u64 q;\n\t.reg .u32 l, h;\n\t"
