@@ -97,7 +97,9 @@ count_kernel(const uint32_t *__restrict__ u, uint64_t n, uint64_t s_begin, uint6
 //      all 512 spacings
 // What it costs is shared-memory wavefronts (about 450 per sample, against
 // some 6000 cycles of two bitonic sorts with a barrier per stage, one day per
-// thread).  At 65536 x 4096 on GB300 the whole battery call took 12.0 ms with
+// thread); the ranks packed four bits each and the byte counts in shared memory
+// keep it within 64 registers (spilled words went to L2 past the shared memory:
+// 1.24 ms).  At 65536 x 4096 on GB300 the whole battery call took 12.0 ms with
 // those sorts and takes 1.24 ms with this kernel.
 // Inputs that are not spread (a bucket of 16 days or more, more than 32
 // candidates) take repeats_by_sorting, so no input costs more than before.
@@ -166,53 +168,64 @@ __device__ __noinline__ int repeats_by_sorting(uint32_t *v, const uint32_t *src,
     return __reduce_add_sync(kAllLanes, r);
 }
 
+// Where byte value b's count is kept: lane l adds those of bytes 4 l + i and
+// 128 + 4 l + i, and its neighbours' lie beside them.
+__device__ __forceinline__ int byte_at(int b)
+{
+    return 32 * (4 * (b >> 7) + (b & 3)) + (b >> 2 & 31);
+}
+
 // Repeated spacings of the sample whose words are col[shift .. shift + 512)
 // (col is overwritten), or -1 when the days are not spread.  scratch: its
 // first 256 words zero on entry, and on exit unless -1 is returned.  Adds the
-// sample's top-byte counts to bins (lane l: bytes 4 l + i and 128 + 4 l + i),
-// or, when a bucket is too full for them, to `bytes`.
+// sample's top-byte counts to `bytes` (byte_at).
 __device__ __forceinline__ int repeats(uint32_t *scratch, uint32_t *col, int shift, int lane,
-                                       uint32_t (&bins)[8], uint32_t *bytes)
+                                       uint32_t *bytes)
 {
     constexpr int P = kDays / 32;
     const uint32_t below = (1u << lane) - 1;
     uint4 *const quad = reinterpret_cast<uint4 *>(scratch);
-    uint32_t u[P], place[P];
+    uint32_t u[P];
 #pragma unroll
     for (int i = 0; i < P; ++i)
         u[i] = col[shift + lane + 32 * i];
-    // bucket u >> 22: counter word u >> 24, bits 8 * (bucket % 4) up
+    // bucket u >> 22: counter word u >> 24, bits 8 * (bucket % 4) up; the ranks
+    // are kept four bits each
+    uint32_t rank[2] = {0, 0}, most = 0;
 #pragma unroll
-    for (int i = 0; i < P; ++i)
-        place[i] = atomicAdd(&scratch[u[i] >> 24], 1u << ((u[i] >> 22 << 3) & 31));
-    uint32_t most = 0;
+    for (int h = 0; h < 2; ++h) {
+        uint32_t old[P / 2];
 #pragma unroll
-    for (int i = 0; i < P; ++i) {
-        place[i] = (place[i] >> ((u[i] >> 22 << 3) & 31)) & 255u;
-        most = max(most, place[i]);
+        for (int i = 0; i < P / 2; ++i) {
+            const uint32_t v = u[h * (P / 2) + i];
+            old[i] = atomicAdd(&scratch[v >> 24], 1u << ((v >> 22 << 3) & 31));
+        }
+#pragma unroll
+        for (int i = 0; i < P / 2; ++i) {
+            const uint32_t r = (old[i] >> ((u[h * (P / 2) + i] >> 22 << 3) & 31)) & 255u;
+            most = max(most, r);
+            rank[h] |= r << (4 * i);  // spilt over only when `most` is 15 or more
+        }
     }
     most = __reduce_max_sync(kAllLanes, most);
     __syncwarp();
     if (most >= kMostInBucket) {  // the counters may have overflowed
 #pragma unroll
         for (int i = 0; i < P; ++i)
-            atomicAdd(&bytes[u[i] >> 24], 1u);
+            atomicAdd(&bytes[byte_at(u[i] >> 24)], 1u);
         return -1;
     }
     {
         const uint4 lo = quad[lane], hi = quad[32 + lane];
         const uint32_t c[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-        uint32_t incl[8], first[8], total[2] = {0, 0};
+        constexpr uint32_t kSums = 0x01010101u;  // byte k of c * kSums: counters 0 .. k
+        uint32_t both = 0;  // both halves' totals: counts stay below 2^16
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            incl[i] = c[i] * 0x01010101u;  // byte k: the word's counters 0 .. k
-            const uint32_t sum = incl[i] >> 24;
-            bins[i] += sum;
-            first[i] = total[i >> 2];
-            total[i >> 2] += sum;
+            const uint32_t sum = c[i] * kSums >> 24;
+            atomicAdd(&bytes[32 * i + lane], sum);
+            both += sum << (i < 4 ? 0 : 16);
         }
-        // both halves' scans in one: counts stay below 2^16
-        const uint32_t both = total[0] | total[1] << 16;
         uint32_t s = both;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -222,30 +235,32 @@ __device__ __forceinline__ int repeats(uint32_t *scratch, uint32_t *col, int shi
         }
         const uint32_t low_half = __shfl_sync(kAllLanes, s, 31) & 0xFFFFu;
         s -= both;
-        const uint32_t before[2] = {s & 0xFFFFu, (s >> 16) + low_half};
         uint4 *const first_of = reinterpret_cast<uint4 *>(scratch + kFirstPlaces);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            uint32_t w[8];
+            uint32_t before = h == 0 ? s & 0xFFFFu : (s >> 16) + low_half;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const uint32_t excl = incl[4 * h + i] - c[4 * h + i];
-                const uint32_t base = (first[4 * h + i] + before[h]) * 0x10001u;
-                w[2 * i] = __byte_perm(excl, 0, 0x4140) + base;  // 16-bit places
-                w[2 * i + 1] = __byte_perm(excl, 0, 0x4342) + base;
+            for (int i = 0; i < 4; i += 2) {
+                uint32_t w[4];
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const uint32_t incl = c[4 * h + i + j] * kSums;
+                    const uint32_t excl = incl - c[4 * h + i + j], base = before * 0x10001u;
+                    w[2 * j] = __byte_perm(excl, 0, 0x4140) + base;  // 16-bit places
+                    w[2 * j + 1] = __byte_perm(excl, 0, 0x4342) + base;
+                    before += incl >> 24;
+                }
+                first_of[64 * h + 2 * lane + i / 2] = make_uint4(w[0], w[1], w[2], w[3]);
             }
-            first_of[64 * h + 2 * lane] = make_uint4(w[0], w[1], w[2], w[3]);
-            first_of[64 * h + 2 * lane + 1] = make_uint4(w[4], w[5], w[6], w[7]);
         }
     }
     __syncwarp();
     const uint16_t *const first_of = reinterpret_cast<const uint16_t *>(scratch + kFirstPlaces);
 #pragma unroll
-    for (int i = 0; i < P; ++i)
-        place[i] += first_of[u[i] >> 22];
-#pragma unroll
-    for (int i = 0; i < P; ++i)
-        col[place[i] + ((place[i] & ~15u) >> 2)] = u[i] >> 8;
+    for (int i = 0; i < P; ++i) {
+        const uint32_t place = first_of[u[i] >> 22] + (rank[i / (P / 2)] >> (4 * (i % (P / 2))) & 15u);
+        col[place + ((place & ~15u) >> 2)] = u[i] >> 8;
+    }
     __syncwarp();
 #pragma unroll
     for (int i = 0; i < kScratch / 128; ++i)  // the bit map
@@ -348,7 +363,6 @@ sample_kernel(const uint32_t *__restrict__ u, uint64_t n, uint32_t samples, Devi
     if (t == 0)
         S.ones = 0;
     uint32_t ones = 0;  // at most 512 per pass, below 2^21 / 16 passes
-    uint32_t bins[8] = {};
     const int c = lane & (kSampleWarps - 1);
     const int row = 32 * warp + R * (lane >> 4);
     auto sample_at = [&](uint32_t q) {  // its first word
@@ -377,7 +391,7 @@ sample_kernel(const uint32_t *__restrict__ u, uint64_t n, uint32_t samples, Devi
         }
         __syncthreads();
         if (q0 + warp < samples) {
-            int r = repeats(S.scratch[warp], S.column[warp], warp, lane, bins, S.bytes);
+            int r = repeats(S.scratch[warp], S.column[warp], warp, lane, S.bytes);
             if (r < 0) {
                 __syncwarp();
                 r = repeats_by_sorting(S.scratch[warp], sample_at((uint32_t)q0 + warp), n, lane);
@@ -391,12 +405,9 @@ sample_kernel(const uint32_t *__restrict__ u, uint64_t n, uint32_t samples, Devi
         }
     }
     atomicAdd(&S.ones, (unsigned long long)ones);
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-        atomicAdd(&S.bytes[128 * (i >> 2) + 4 * lane + (i & 3)], bins[i]);
     __syncthreads();
     if (t < 256) {
-        atomicAdd(&out->bytes[t], (unsigned long long)S.bytes[t]);
+        atomicAdd(&out->bytes[t], (unsigned long long)S.bytes[byte_at(t)]);
         atomicAdd(&out->serial[t], (unsigned long long)S.serial[t]);
     }
     if (t < 16 && S.birthday[t])
