@@ -283,7 +283,8 @@ typedef struct rng_battery_counts {
  * (DEVICE, uint32, 4-byte aligned) holds n_per_stream rows of n_streams
  * outputs, output j of stream s at dev_u[j * n_streams + s] (rng_generate's
  * layout); the counts go to *host_counts (HOST).  Runs on cuda_stream and
- * SYNCHRONISES it; allocates a few KB of device memory for the call.
+ * SYNCHRONISES it; allocates a few KB of device memory for the call when more
+ * than eight calls run on the device at once.
  * Errors: RNG_ERR_ARG, RNG_ERR_OOM, RNG_ERR_CUDA.
  * Paper: the generators' randomness is assessed with DIEHARD and TestU01
  * (Sec. "Performance evaluation"); these four tests come from those

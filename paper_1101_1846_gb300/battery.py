@@ -80,10 +80,10 @@ def counts(u: torch.Tensor, n_streams: int, n_per_stream: int,
                                       ctypes.byref(c), ctypes.c_void_p(s.cuda_stream)),
                "rng_battery")
     return {"n_outputs": int(c.n_outputs), "ones": int(c.ones),
-            "bytes": np.array(c.bytes[:], dtype=np.uint64),
-            "serial": np.array(c.serial[:], dtype=np.uint64),
+            "bytes": np.array(c.bytes, dtype=np.uint64),
+            "serial": np.array(c.serial, dtype=np.uint64),
             "birthday_samples": int(c.birthday_samples),
-            "birthday": np.array(c.birthday[:], dtype=np.uint64)}
+            "birthday": np.array(c.birthday, dtype=np.uint64)}
 
 
 def _chi2_sf(x: float, dof: int) -> float:

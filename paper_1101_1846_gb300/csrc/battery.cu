@@ -19,6 +19,7 @@
 // histograms of the outputs that belong to no sample (rows past the last
 // multiple of 512, and streams past the cap).
 #include <algorithm>
+#include <atomic>
 
 #include "gbrng.cuh"
 
@@ -416,6 +417,42 @@ sample_kernel(const uint32_t *__restrict__ u, uint64_t n, uint32_t samples, Devi
         atomicAdd(&out->ones, S.ones);
 }
 
+// Device counts of the calls in progress: a few fixed ones per device, so that
+// a call need not allocate and free (about 30 us, and the free waits for the
+// device); further calls at once, from other host threads, allocate.
+constexpr int kSlots = 8, kMaxDevices = 64;
+__device__ DeviceCounts g_slots[kSlots];
+std::atomic<bool> g_taken[kMaxDevices][kSlots];
+
+// One call's counts, given back when the call returns (it has synchronised).
+struct Scratch {
+    DeviceCounts *counts = nullptr;
+    std::atomic<bool> *taken = nullptr;  // nullptr: allocated
+
+    DeviceCounts *take()
+    {
+        int dev = -1;
+        void *base = nullptr;
+        if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices &&
+            cudaGetSymbolAddress(&base, g_slots) == cudaSuccess)
+            for (int i = 0; i < kSlots; ++i)
+                if (!g_taken[dev][i].exchange(true)) {
+                    taken = &g_taken[dev][i];
+                    return counts = static_cast<DeviceCounts *>(base) + i;
+                }
+        if (cudaMalloc(&counts, sizeof(DeviceCounts)) != cudaSuccess)
+            counts = nullptr;
+        return counts;
+    }
+    ~Scratch()
+    {
+        if (taken)
+            taken->store(false);
+        else
+            cudaFree(counts);
+    }
+};
+
 // Counts rows [row0, row1) of streams [s_begin, n).
 int launch_count(const uint32_t *u, uint64_t n, uint64_t s_begin, uint64_t row0, uint64_t row1,
                  DeviceCounts *d, cudaStream_t st)
@@ -465,8 +502,9 @@ extern "C" int rng_battery(const void *dev_u, uint64_t n_streams, uint64_t n_per
         return set_error(RNG_ERR_ARG);
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const uint32_t *u = static_cast<const uint32_t *>(dev_u);
-    DeviceCounts *d = nullptr;
-    if (cudaMalloc(&d, sizeof(DeviceCounts)) != cudaSuccess)
+    Scratch scratch;
+    DeviceCounts *const d = scratch.take();
+    if (!d)
         return set_error(RNG_ERR_OOM);
     int status = cuda_status(cudaMemsetAsync(d, 0, sizeof(DeviceCounts), st));
     const uint64_t blocks = n_per_stream / kDays;
@@ -489,9 +527,10 @@ extern "C" int rng_battery(const void *dev_u, uint64_t n_streams, uint64_t n_per
         status = cuda_status(cudaMemcpyAsync(&h, d, sizeof(h), cudaMemcpyDeviceToHost, st));
     if (!status)
         status = cuda_status(cudaStreamSynchronize(st));
-    cudaFree(d);
-    if (status)
+    if (status) {
+        cudaStreamSynchronize(st);  // nothing writes the counts when they are given back
         return status;
+    }
     host_counts->n_outputs = n_streams * n_per_stream;
     host_counts->ones = h.ones;
     for (int k = 0; k < 256; ++k) {

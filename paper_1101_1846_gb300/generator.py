@@ -11,8 +11,10 @@ from . import capi
 
 
 def _stream_ptr(stream: torch.cuda.Stream | None) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    if stream is not None:
+        return int(stream.cuda_stream)
+    # torch.cuda.current_stream().cuda_stream without the Stream object
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _dtype(fmt: int) -> torch.dtype:
@@ -35,6 +37,7 @@ class Generator:
         if not h:
             raise capi.RngError(capi.lib().rng_last_error(), "rng_create")
         self.h = h
+        self._lib = capi.lib()
         self.kind = int(kind)
         self.n_streams = int(n_streams)
         self.seed = int(seed)
@@ -60,8 +63,7 @@ class Generator:
         self.close()
 
     def _bind(self, stream) -> None:
-        capi.check(capi.lib().rng_set_stream(self.h, ctypes.c_void_p(_stream_ptr(stream))),
-                   "rng_set_stream")
+        capi.check(self._lib.rng_set_stream(self.h, _stream_ptr(stream)), "rng_set_stream")
 
     def generate(self, n_per_stream: int, fmt: int | str = capi.RNG_U32,
                  out: torch.Tensor | None = None,
@@ -73,8 +75,7 @@ class Generator:
         assert out.is_cuda and out.is_contiguous() and out.element_size() == 4
         assert out.numel() >= n_per_stream * self.n_streams
         self._bind(stream)
-        capi.check(capi.lib().rng_generate(self.h, n_per_stream,
-                                           ctypes.c_void_p(out.data_ptr()), fmt),
+        capi.check(self._lib.rng_generate(self.h, n_per_stream, out.data_ptr(), fmt),
                    "rng_generate")
         return out
 
@@ -90,8 +91,8 @@ class Generator:
             assert offset + (n_per_stream - 1) * ld + count <= out.numel()
         self._bind(stream)
         ptr = out.data_ptr() + 4 * offset
-        capi.check(capi.lib().rng_generate_range(self.h, s_begin, s_end, n_per_stream,
-                                                 ctypes.c_void_p(ptr), ld, fmt),
+        capi.check(self._lib.rng_generate_range(self.h, s_begin, s_end, n_per_stream, ptr, ld,
+                                                fmt),
                    "rng_generate_range")
 
     def generate_host(self, n_per_stream: int, fmt: int | str = capi.RNG_U32,
@@ -124,8 +125,8 @@ class Generator:
         assert out.is_cuda and out.is_contiguous() and out.element_size() == 8
         assert out.numel() >= self.n_streams
         self._bind(stream)
-        capi.check(capi.lib().rng_generate_reduce(self.h, n_per_stream, int(op),
-                                                  ctypes.c_void_p(out.data_ptr())),
+        capi.check(self._lib.rng_generate_reduce(self.h, n_per_stream, int(op),
+                                                 out.data_ptr()),
                    "rng_generate_reduce")
         return out
 
@@ -133,7 +134,7 @@ class Generator:
         """Advances every stream by k steps without producing the outputs
         in between (rng_jump)."""
         self._bind(stream)
-        capi.check(capi.lib().rng_jump(self.h, int(k) & (2**64 - 1)), "rng_jump")
+        capi.check(self._lib.rng_jump(self.h, int(k) & (2**64 - 1)), "rng_jump")
 
     def device_view(self) -> capi.rng_device_view:
         v = capi.rng_device_view()
