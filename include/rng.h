@@ -351,8 +351,10 @@ typedef struct rng_plan *rng_plan_handle;
  * the work list is copied to the device (synchronises).  threads = CTA size
  * (power of two, 32..512; 0 = 512), ctas_per_sm = resident CTAs the
  * persistent grid puts on each SM (1..32; 0 = as many as fit); both 0 = the
- * default shape, CTAs of 512 threads, one per SM (the fastest measured on
- * GB300).  With ctas_per_sm = 1 the launch reserves more than half an SM's
+ * default shape, the fastest measured on GB300 for what the list holds: CTAs
+ * of 512 threads, one per SM, or for few tiles CTAs of 64, two or four per SM
+ * (a refill gives such a plan CTAs of 512).  With ctas_per_sm = 1 the launch
+ * reserves more than half an SM's
  * shared memory (unused) so that no SM takes a second CTA.  Items of the
  * same handle must cover disjoint stream ranges (they then run side by
  * side); items with n_per_stream = 0 are
@@ -393,7 +395,8 @@ int rng_plan_launch(rng_plan_handle p, void *cuda_stream);
 int rng_plan_refill(rng_plan_handle p, const rng_batch_item *items, size_t n_items,
                     void *cuda_stream);
 
-/* Tiles in the plan, and its CTA size and persistent grid size. */
+/* Tiles in the plan's current list, and its CTA size and persistent grid
+ * size. */
 uint64_t rng_plan_tiles(rng_plan_handle p);
 int rng_plan_shape(rng_plan_handle p, int *threads, int *grid);
 

@@ -201,8 +201,9 @@ void launch_mixed(int kind, int grid, int threads, bool one_per_sm, cudaStream_t
     fn<<<grid, threads, smem, st>>>(units, n_units, next);
 }
 
-// Plan shape when the caller passes 0 for both: CTAs of 512 threads, one per
-// SM.  Measured on GB300 with the 10,000-instance workload (256-row pieces):
+// Plan shape when the caller passes 0 for both, by what the list holds
+// (choose_shape).  Lists of many tiles: CTAs of 512 threads, one per SM.
+// Measured on GB300 with the 10,000-instance workload (256-row pieces):
 // 914 GSamples/s with 128 threads (as many CTAs as fit), about 1570 with 512
 // (two per SM); then, on one box, 1605 with two CTAs of 512 per SM, 1641
 // with one (1632 with the grid alone keeping to one, without the
@@ -210,6 +211,44 @@ void launch_mixed(int kind, int grid, int threads, bool one_per_sm, cudaStream_t
 // 1631 with two, 1664 with one.
 constexpr int kDefaultThreads = 512;
 constexpr int kDefaultCtas = 1;
+
+// Lists of few tiles end with their longest tile, whose rows follow one
+// another faster the fewer warps its SM runs, and they share the SMs more
+// evenly in small tiles: CTAs of 64 threads, two to an SM where some item is
+// long, four where none is (a short tile waits for its state more than for the
+// pipes).  A refill, which a caller runs before every launch, keeps the larger
+// tiles: writing eight times as many took 48 served requests of mixed sizes from
+// 609 to 707 us, most of it host time.  GB300, us a launch, by tiles of 128 threads (4 x 128 streams):
+//                                                        512 x 1  64 x 2  64 x 4
+//     20: 16 items of up to 1174 streams, 400 rows          56.2    27.4    31.1
+//    357: 216 of up to 2268, 1018                          137.6    64.4    81.0
+//    552: 40 of up to 43,000, 16                            13.2    13.8    11.5
+//    612: 40 of up to 43,000, 250                           52.0    31.3    29.9
+//    622: 462 of up to 1064, 820                           141.3    65.7    82.8
+//   1068: 500 of up to 4000, 1000                          187.8    84.7   111.8
+//   1160: 60 of up to 43,000, 250                           43.8    52.8    40.3
+//   1203: 80 of up to 65,536, 1024                         146.6    97.6   119.2
+//   1740: 512 of up to 8000, 500                           101.3    88.4    81.3
+//   1833: 119 of up to 43,400, 87                           37.5    46.3    33.6
+//   2603: 512 of up to 12,000, 1024                        228.2   226.5   230.9
+//   3666: 200 of up to 65,536, 1024                        312.6   364.2   360.0
+//   8787: 512 of up to 65,536, 1024                        719.4   837.4   819.6
+constexpr int kFewThreads = 64;
+constexpr uint64_t kFewTiles = 13;      // per SM: up to here CTAs of 64 threads
+constexpr uint64_t kFewLongTiles = 8;   // per SM: up to here two of them to an SM,
+constexpr uint64_t kFewLongRows = 384;  // when an item has this many rows
+struct Shape {
+    int threads, ctas_per_sm;
+};
+
+Shape shape_for(uint64_t tiles_of_128, uint64_t longest, int sms)
+{
+    if (tiles_of_128 > kFewTiles * sms)
+        return Shape{kDefaultThreads, kDefaultCtas};
+    const bool slow = tiles_of_128 <= kFewLongTiles * sms && longest >= kFewLongRows;
+    return Shape{kFewThreads, slow ? 2 : 4};
+}
+
 constexpr int kHint = 1;  // streaming stores, as the plain kernels
 
 // An item's stream range and row stride with the defaults filled in.
@@ -336,6 +375,19 @@ void order_units(Unit *u, uint64_t n)
     });
 }
 
+uint64_t longest_of(const rng_batch_item *items, size_t n_items)
+{
+    uint64_t rows = 0;
+    for (size_t i = 0; i < n_items; ++i)
+        rows = std::max<uint64_t>(rows, items[i].n_per_stream);
+    return rows;
+}
+
+Shape choose_shape(const rng_batch_item *items, size_t n_items, int sms)
+{
+    return shape_for(fill_units(items, n_items, 128, nullptr, 0), longest_of(items, n_items), sms);
+}
+
 int grid_for(int device, int threads, int ctas_per_sm, int *grid, bool mixed = false)
 {
     int sms = 0, fit = 0;
@@ -360,6 +412,7 @@ struct Plan {
     unsigned long long *d_next = nullptr;
     int threads = kDefaultThreads;
     int grid = 0;
+    Shape refills{kDefaultThreads, kDefaultCtas};  // the shape a refill gives the plan
     std::vector<Claim> claims;       // refill overlap check
     // refill staging: two pinned host lists used in turn, so that the copy
     // to the device is a plain DMA and the call does not wait for it; a
@@ -375,6 +428,7 @@ struct Plan {
     int mixed_kind = 0;  // their kind (one per mapped refill)
     int ctas_per_sm = 0;
     int grid_mixed = 0;
+    int grid_refill = 0;  // of plain refills, 0 before the first
     uint32_t *d_maps = nullptr;
     uint64_t cap_maps = 0;  // words
     uint32_t *pinned_maps[2] = {nullptr, nullptr};
@@ -411,8 +465,7 @@ extern "C" rng_plan_handle rng_plan_create(const rng_batch_item *items, size_t n
         set_error(RNG_ERR_ARG);
         return nullptr;
     }
-    if (threads == 0 && ctas_per_sm == 0)
-        ctas_per_sm = kDefaultCtas;
+    const bool choose = threads == 0 && ctas_per_sm == 0;
     if (threads == 0)
         threads = kDefaultThreads;
     if (threads < 32 || threads > 512 || (threads & (threads - 1)) || ctas_per_sm < 0 ||
@@ -424,6 +477,14 @@ extern "C" rng_plan_handle rng_plan_create(const rng_batch_item *items, size_t n
     std::vector<Claim> claims(n_items);
     if (validate_items(items, n_items, claims.data(), &device))
         return nullptr;
+    if (choose) {
+        int sms = 0;
+        if (cuda_status(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device)))
+            return nullptr;
+        const Shape s = choose_shape(items, n_items, sms);
+        threads = s.threads;
+        ctas_per_sm = s.ctas_per_sm;
+    }
     std::vector<Unit> units(fill_units(items, n_items, threads, nullptr, 0));
     fill_units(items, n_items, threads, units.data(), units.size());
     order_units(units.data(), units.size());
@@ -438,6 +499,7 @@ extern "C" rng_plan_handle rng_plan_create(const rng_batch_item *items, size_t n
         p->device = device;
         p->threads = threads;
         p->ctas_per_sm = ctas_per_sm;
+        p->refills = choose ? Shape{kDefaultThreads, kDefaultCtas} : Shape{threads, ctas_per_sm};
         p->n_units = units.size();
         st = grid_for(device, threads, ctas_per_sm, &p->grid);
     }
@@ -555,7 +617,9 @@ int refill(Plan *p, const rng_batch_item *items, size_t n_items, const uint64_t 
                 return set_error(RNG_ERR_ARG);
             kind = k;
         }
-    const uint64_t n = fill_units(items, n_items, p->threads, nullptr, 0);
+    const Shape shape = p->refills;
+    const uint64_t n = fill_units(items, n_items, shape.threads, nullptr, 0);
+    int grid = maps ? p->grid_mixed : p->grid_refill;
     int prev = -1;
     cudaGetDevice(&prev);
     if (prev != p->device)
@@ -575,8 +639,6 @@ int refill(Plan *p, const rng_batch_item *items, size_t n_items, const uint64_t 
                            p->pinned_maps_cap[k ^ 1]);
         if (!st)
             st = ensure_device(&p->d_maps, &p->cap_maps, map_words, stream);
-        if (!st && !p->grid_mixed)
-            st = grid_for(p->device, p->threads, p->ctas_per_sm, &p->grid_mixed, true);
         if (!st) {
             dmaps.resize(n_items);
             for (size_t i = 0; i < n_items; ++i)
@@ -587,8 +649,10 @@ int refill(Plan *p, const rng_batch_item *items, size_t n_items, const uint64_t 
                                              cudaMemcpyHostToDevice, stream));
         }
     }
+    if (!st && !grid)
+        st = grid_for(p->device, shape.threads, shape.ctas_per_sm, &grid, maps != nullptr);
     if (!st)
-        fill_units(items, n_items, p->threads, p->pinned[k], n, maps ? dmaps.data() : nullptr);
+        fill_units(items, n_items, shape.threads, p->pinned[k], n, maps ? dmaps.data() : nullptr);
     if (!st && n)
         st = cuda_status(cudaMemcpyAsync(p->d_units, p->pinned[k], n * sizeof(Unit),
                                          cudaMemcpyHostToDevice, stream));
@@ -596,6 +660,12 @@ int refill(Plan *p, const rng_batch_item *items, size_t n_items, const uint64_t 
         st = cuda_status(cudaEventRecord(p->copied[k], stream));
     if (!st) {
         p->n_units = n;
+        p->threads = shape.threads;
+        p->ctas_per_sm = shape.ctas_per_sm;
+        if (maps)
+            p->grid_mixed = grid;
+        else
+            p->grid = p->grid_refill = grid;
         p->mixed = maps != nullptr;
         p->mixed_kind = kind;
         p->turn ^= 1;
@@ -699,6 +769,22 @@ void *g_noalloc_dev_ptr[64] = {nullptr};         // device address of the scratc
 Unit g_noalloc_host_units[kNoAllocMaxTiles];     // host copy of the work list
 Claim g_noalloc_claims[kNoAllocMaxItems];       // overlap check
 
+// CTAs of 128 threads per SM.  The capacity above fixes the tiles, so the
+// list chooses the grid alone: one where a list of few tiles has a long item,
+// else two.  GB300, us, with one / two / four / as many as fit (tiles):
+//    357: 216 items of up to 2268 streams, 1018 rows    64 /   84 /  136 /  176
+//   1068: 500 of up to 4000, 1000                      103 /  111 /  202 /  331
+//   1833: 119 of up to 43,400, 87                       52 /   37 /   42 /   51
+//   8787: 512 of up to 65,536, 1024                    894 /  761 /  910 / 1137
+int noalloc_ctas(const rng_batch_item *items, size_t n_items, uint64_t n_units, int device)
+{
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
+        return 0;  // grid_for reports it
+    const bool slow = n_units <= kFewLongTiles * sms && longest_of(items, n_items) >= kFewLongRows;
+    return slow ? 1 : 2;
+}
+
 }  // namespace
 }  // namespace gbrng
 
@@ -742,7 +828,7 @@ extern "C" int rng_generate_batch_noalloc(const rng_batch_item *items, size_t n_
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     int grid = 0;
     if (!st)
-        st = grid_for(device, threads, 0, &grid);
+        st = grid_for(device, threads, noalloc_ctas(items, n_items, n_units, device), &grid);
     unsigned char *base = static_cast<unsigned char *>(g_noalloc_dev_ptr[device]);
     unsigned long long *next = reinterpret_cast<unsigned long long *>(base);
     Unit *units = reinterpret_cast<Unit *>(base + kNoAllocHeader);
