@@ -353,7 +353,7 @@ typedef struct rng_plan *rng_plan_handle;
  * persistent grid puts on each SM (1..32; 0 = as many as fit); both 0 = the
  * default shape, the fastest measured on GB300 for what the list holds: CTAs
  * of 512 threads, one per SM, or for few tiles CTAs of 64, two or four per SM
- * (a refill gives such a plan CTAs of 512).  With ctas_per_sm = 1 the launch
+ * (a refill of such a plan: CTAs of 512 or 128, one per SM).  With ctas_per_sm = 1 the launch
  * reserves more than half an SM's
  * shared memory (unused) so that no SM takes a second CTA.  Items of the
  * same handle must cover disjoint stream ranges (they then run side by
@@ -516,8 +516,9 @@ int rng_server_stats(rng_server_handle s, uint64_t *out8);
 int rng_server_set_tick_bytes(rng_server_handle s, uint64_t bytes);
 
 /* Shape of the engine's persistent kernel, as rng_plan_create's `threads`
- * (a power of two in [32, 512]; default 512) and `ctas_per_sm` (0 = as many
- * as fit; default 1).  Synchronises the engine's streams if ticks have run;
+ * (a power of two in [32, 512]) and `ctas_per_sm` (0 = as many as fit); until
+ * it is called each tick takes CTAs of 512 or 128 threads, one per SM, by what
+ * it holds.  Synchronises the engine's streams if ticks have run;
  * the next tick of each lane uses the new shape.  Output is the same for any shape.
  * RNG_ERR_ARG outside those ranges. */
 int rng_server_set_plan_shape(rng_server_handle s, int threads, int ctas_per_sm);

@@ -216,9 +216,7 @@ constexpr int kDefaultCtas = 1;
 // another faster the fewer warps its SM runs, and they share the SMs more
 // evenly in small tiles: CTAs of 64 threads, two to an SM where some item is
 // long, four where none is (a short tile waits for its state more than for the
-// pipes).  A refill, which a caller runs before every launch, keeps the larger
-// tiles: writing eight times as many took 48 served requests of mixed sizes from
-// 609 to 707 us, most of it host time.  GB300, us a launch, by tiles of 128 threads (4 x 128 streams):
+// pipes).  GB300, us a launch, by tiles of 128 threads (4 x 128 streams):
 //                                                        512 x 1  64 x 2  64 x 4
 //     20: 16 items of up to 1174 streams, 400 rows          56.2    27.4    31.1
 //    357: 216 of up to 2268, 1018                          137.6    64.4    81.0
@@ -388,6 +386,25 @@ Shape choose_shape(const rng_batch_item *items, size_t n_items, int sms)
     return shape_for(fill_units(items, n_items, 128, nullptr, 0), longest_of(items, n_items), sms);
 }
 
+// A refill, which a caller runs before every launch, pays for its tiles on the
+// host: it takes CTAs of 128 threads where the list is short and its rows are
+// many, else of 512, one per SM in both.  GB300, us from submission to the last
+// sample of a serving burst, 512 / 256 / 128 threads (tiles of 128 a lane, rows
+// of the largest request): 6 clients of 14,668 streams (87, 822) 612 / 511 / 422,
+// 8 of 5371 (44, 581) 573 / 475 / 447, 6 of 50,632 (297, 90) 138 / 122 / 117, 52
+// of 12,111 (624, 34) 70 / 68 / 66, 64 of 65,536 (4096, 256) 142 / 144 / 163.
+// Plans alone, 16 rows, 552 tiles: 13.2 us with 512, 15.0 with 128; 250 rows, 612
+// tiles: 52 and 34; 1018 rows, 357 tiles: 138 and 64.
+constexpr uint64_t kRefillTiles = 5;    // per SM
+constexpr uint64_t kRefillRows = 128;
+
+Shape refill_shape(const rng_batch_item *items, size_t n_items, int sms)
+{
+    const bool few = longest_of(items, n_items) >= kRefillRows &&
+                     fill_units(items, n_items, 128, nullptr, 0) <= kRefillTiles * sms;
+    return Shape{few ? 128 : kDefaultThreads, 1};
+}
+
 int grid_for(int device, int threads, int ctas_per_sm, int *grid, bool mixed = false)
 {
     int sms = 0, fit = 0;
@@ -412,7 +429,7 @@ struct Plan {
     unsigned long long *d_next = nullptr;
     int threads = kDefaultThreads;
     int grid = 0;
-    Shape refills{kDefaultThreads, kDefaultCtas};  // the shape a refill gives the plan
+    int sms = 0;  // the lists choose their shapes; 0 = the caller's holds
     std::vector<Claim> claims;       // refill overlap check
     // refill staging: two pinned host lists used in turn, so that the copy
     // to the device is a plain DMA and the call does not wait for it; a
@@ -428,7 +445,6 @@ struct Plan {
     int mixed_kind = 0;  // their kind (one per mapped refill)
     int ctas_per_sm = 0;
     int grid_mixed = 0;
-    int grid_refill = 0;  // of plain refills, 0 before the first
     uint32_t *d_maps = nullptr;
     uint64_t cap_maps = 0;  // words
     uint32_t *pinned_maps[2] = {nullptr, nullptr};
@@ -477,8 +493,8 @@ extern "C" rng_plan_handle rng_plan_create(const rng_batch_item *items, size_t n
     std::vector<Claim> claims(n_items);
     if (validate_items(items, n_items, claims.data(), &device))
         return nullptr;
+    int sms = 0;
     if (choose) {
-        int sms = 0;
         if (cuda_status(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device)))
             return nullptr;
         const Shape s = choose_shape(items, n_items, sms);
@@ -499,7 +515,7 @@ extern "C" rng_plan_handle rng_plan_create(const rng_batch_item *items, size_t n
         p->device = device;
         p->threads = threads;
         p->ctas_per_sm = ctas_per_sm;
-        p->refills = choose ? Shape{kDefaultThreads, kDefaultCtas} : Shape{threads, ctas_per_sm};
+        p->sms = sms;
         p->n_units = units.size();
         st = grid_for(device, threads, ctas_per_sm, &p->grid);
     }
@@ -617,9 +633,11 @@ int refill(Plan *p, const rng_batch_item *items, size_t n_items, const uint64_t 
                 return set_error(RNG_ERR_ARG);
             kind = k;
         }
-    const Shape shape = p->refills;
+    const Shape shape = p->sms ? refill_shape(items, n_items, p->sms)
+                               : Shape{p->threads, p->ctas_per_sm};
     const uint64_t n = fill_units(items, n_items, shape.threads, nullptr, 0);
-    int grid = maps ? p->grid_mixed : p->grid_refill;
+    // one CTA per SM always fits
+    int grid = p->sms ? p->sms : maps ? p->grid_mixed : p->grid;
     int prev = -1;
     cudaGetDevice(&prev);
     if (prev != p->device)
@@ -662,10 +680,8 @@ int refill(Plan *p, const rng_batch_item *items, size_t n_items, const uint64_t 
         p->n_units = n;
         p->threads = shape.threads;
         p->ctas_per_sm = shape.ctas_per_sm;
-        if (maps)
-            p->grid_mixed = grid;
-        else
-            p->grid = p->grid_refill = grid;
+        p->grid_mixed = maps ? grid : p->grid_mixed;
+        p->grid = !maps || p->sms ? grid : p->grid;
         p->mixed = maps != nullptr;
         p->mixed_kind = kind;
         p->turn ^= 1;

@@ -1,7 +1,7 @@
-"""The default shape of batched plans (choose_shape in csrc/batch.cu): lists
-on both sides of each line of the rule, launched, refilled (which gives the plan
-its large shape), and through the allocation-free entry point, give what plain calls of
-the same generators give, bit for bit, and leave the same states."""
+"""The shapes that plans choose by what they hold (choose_shape and
+refill_shape in csrc/batch.cu): lists on both sides of each line of the rules,
+launched, refilled and through the allocation-free entry point, give what
+plain calls of the same generators give, bit for bit."""
 from __future__ import annotations
 
 import pytest
@@ -71,18 +71,31 @@ def test_shapes_equal_plain_calls(per_sm, over, rows, shape):
     x.check()
 
 
-def test_refills_return_to_the_large_shape():
+def test_refills_choose_their_shape():
     sm = sms()
     x = Lists(sizes_of(13 * sm + 1))
     plan = Plan(x.take(17, range(10)))
     assert plan.shape == (64, 4 * sm)
     plan.launch()
     x.check()
-    for rows, pick in ((21, range(10)), (385, range(10)), (9, None), (4, [1])):
+    for rows, pick, threads in ((127, range(10), 512), (128, range(10), 128), (9, None, 512),
+                                (385, range(10), 128), (130, None, 512), (4, [1], 512)):
         plan.refill(x.take(rows, pick))
-        assert plan.shape == (512, sm)
+        assert plan.shape == (threads, sm)
         plan.launch()
         x.check()
+
+
+@pytest.mark.parametrize("over,threads", [(0, 128), (1, 512)])
+def test_refill_tile_line(over, threads):
+    x = Lists(sizes_of(5 * sms() + over))
+    plan = Plan(x.take(3))
+    plan.launch()
+    x.check()
+    plan.refill(x.take(128))
+    assert plan.shape == (threads, sms())
+    plan.launch()
+    x.check()
 
 
 def test_explicit_shapes_stay():
