@@ -517,6 +517,59 @@ inline int fit_threads(int threads, uint64_t units)
     return threads;
 }
 
+// CTAs of one size in whole waves of one per SM.  A call of a few waves ends
+// with its last one, which a fixed CTA size leaves nearly empty: 700,000 streams
+// in CTAs of 4096 are 171 CTAs, and 19 of 152 SMs write the second half.  Where
+// less than kEvenFill of the SMs' time is used, the CTAs are made smaller, equal,
+// and as many as whole waves hold.  Every size from one to thirteen waves was
+// timed both ways; above that fill they differ by a few percent either way.
+// GB300, TB/s, fixed and even sizes (r: realigned rows), fill:
+//   KISS u32    668,784 x 470  0.54  4.58  6.45    191,762r x 1640 0.64  4.45  6.11
+//   KISS f32    200,090r x 1572 0.67 3.87  5.67    373,321r x 842  0.62  3.97  5.16
+//   xor128 u32   96,528 x 162  0.62  3.42  4.26    177,530r x 1771 0.59  4.15  6.21
+//   xor128 f32  663,488 x 474  0.53  4.46  7.08    348,553r x 902  0.58  4.06  5.29
+//   XORSHIFT8   197,272 x 1594 0.63  4.29  5.69    338,148r x 930  0.56  3.74  5.01
+//   MWC u32     344,340 x 913  0.57  4.79  6.25    359,769r x 874  0.60  4.95  6.78
+//   MWC f32     641,408 x 490  0.52  4.91  7.13    187,794r x 1675 0.62  4.46  5.95
+constexpr double kEvenFill = 0.8;
+
+// Groups of four streams a CTA of `threads` holds: one a thread, or for
+// realigned rows 31 a warp and one.
+inline uint64_t groups_of(int threads, bool realigned)
+{
+    return realigned ? 31 * (threads / 32) + 1 : threads;
+}
+
+// The CTA size for `groups` groups of four, 0 where CTAs of `per_cta` groups
+// fill their waves.  XORSHIFT8, whose steps take the longest, wants the warps of
+// whole SMs; the others write in denser streams from at most 256 threads, and
+// xor128, whose steps take the shortest, 32-byte rows from 128 (f32 calls of
+// 1.2 GB, TB/s in CTAs of 160-224 and of 96-128: 173,440 streams 4.96 6.07,
+// 195,160 5.68 6.54, 255,048 6.35 6.38).
+inline int even_threads(int kind, uint64_t groups, uint64_t per_cta, bool sectors, bool realigned)
+{
+    const uint64_t ctas = (groups + per_cta - 1) / per_cta;
+    const uint64_t waves = (ctas + kSMs - 1) / kSMs;
+    if (groups <= (uint64_t)kSMs * 128 ||  // at most one warp a scheduler in any case
+        (double)groups >= kEvenFill * (double)(per_cta * kSMs * waves))
+        return 0;
+    const int most = kind == RNG_XORSHIFT8 ? 512 : kind == RNG_XOR128 && sectors ? 128 : 256;
+    for (uint64_t k = 1;; ++k) {
+        const uint64_t each = (groups + kSMs * k - 1) / (kSMs * k);
+        const uint64_t threads = realigned ? 32 * ((each - 1 + 30) / 31) : 32 * ((each + 31) / 32);
+        if (threads <= (uint64_t)most)
+            return (int)std::max<uint64_t>(threads, 32);
+    }
+}
+
+// Whether those CTAs keep an SM to themselves (one_cta_smem): the realigned
+// FP32 kernels, whose conversions wait longer, and XORSHIFT8 run faster beside
+// one another.
+inline bool even_alone(int kind, int fmt, bool realigned)
+{
+    return kind != RNG_XORSHIFT8 && !(realigned && fmt == RNG_F32 && kind != RNG_MWC32);
+}
+
 // V = 2 only for kinds of at most four state words: two groups of the
 // eight-word XORSHIFT8 would not fit the registers of a 512-thread CTA.
 template <int KIND, int FMT>
@@ -644,6 +697,31 @@ int launch_kind(int fmt, const GenLaunch &p, cudaStream_t st)
         sh.v = 1;
         sh.hint = 0;
     }
+    // 16-byte rows and 16-byte state groups: every group of four streams
+    // starts on a 16-byte boundary in the output and in the state words.
+    const bool aligned = (count % 4 == 0) && (p.ld % 4 == 0) && ((uintptr_t)p.out % 16 == 0) &&
+                         (p.n % 4 == 0) && (p.s_begin % 4 == 0) &&
+                         ((uintptr_t)p.state % 16 == 0) &&
+                         (p.a == nullptr || (uintptr_t)p.a % 16 == 0);
+    // whole 32-byte sectors per warp and row: no barriers needed
+    const bool sectors = aligned && (p.ld % 8 == 0) && ((uintptr_t)p.out % 32 == 0);
+    const uint64_t main = count & ~(uint64_t)3;
+    const int sync_threads = fit_threads(kSyncBlock, main / 4);
+    const int vec_threads = fit_threads(sh.block, main / 4 / sh.v);
+    int even = 0;
+    if (!sectors)
+        even = even_threads(KIND, main / 4, groups_of(sync_threads, !aligned), false, !aligned);
+    // KISS with 32-byte rows: FP32 takes CTAs of 128, as many as fit, which even
+    // out by themselves, and so do uint32 CTAs of less than 512 threads (311,776
+    // streams: 6.6 TB/s, 5.4 in three even waves)
+    else if (KIND != RNG_KISS || (fmt == RNG_U32 && vec_threads == sh.block))
+        even = even_threads(KIND, main / 4, sh.hint == 2 ? kTmaThreads : sh.v * vec_threads, true,
+                            false);
+    const bool alone = even && even_alone(KIND, fmt, !aligned);
+    if (even && sectors) {
+        sh.v = 1;
+        sh.hint = sh.hint ? 1 : 0;
+    }
     Fn vec, shift, sync;
     if (fmt == RNG_F32) {
         pick_vec<KIND, RNG_F32>(sh.v, sh.hint, vec);
@@ -654,15 +732,6 @@ int launch_kind(int fmt, const GenLaunch &p, cudaStream_t st)
         shift = sh.hint ? gen_shift<KIND, RNG_U32, 1> : gen_shift<KIND, RNG_U32, 0>;
         sync = sh.hint ? gen_vec_sync<KIND, RNG_U32, 1> : gen_vec_sync<KIND, RNG_U32, 0>;
     }
-    // 16-byte rows and 16-byte state groups: every group of four streams
-    // starts on a 16-byte boundary in the output and in the state words.
-    const bool aligned = (count % 4 == 0) && (p.ld % 4 == 0) && ((uintptr_t)p.out % 16 == 0) &&
-                         (p.n % 4 == 0) && (p.s_begin % 4 == 0) &&
-                         ((uintptr_t)p.state % 16 == 0) &&
-                         (p.a == nullptr || (uintptr_t)p.a % 16 == 0);
-    // whole 32-byte sectors per warp and row: no barriers needed
-    const bool sectors = aligned && (p.ld % 8 == 0) && ((uintptr_t)p.out % 32 == 0);
-    const uint64_t main = count & ~(uint64_t)3;
     uint32_t *out = static_cast<uint32_t *>(p.out);
     Gen *g = p.owner;
     const SplitForm form = aligned ? SplitForm::kAligned : SplitForm::kShifted;
@@ -679,11 +748,11 @@ int launch_kind(int fmt, const GenLaunch &p, cudaStream_t st)
         const uint32_t steps = (uint32_t)std::min<uint64_t>(p.steps - done, 1u << 31);
         uint32_t *o = out + done * p.ld;
         if (aligned && !sectors) {
-            int threads = fit_threads(kSyncBlock, count / 4);
+            const int threads = even ? even : sync_threads;
             uint64_t blocks = (count / 4 + threads - 1) / threads;
             if (blocks > 0x7FFFFFFFull)
                 return set_error(RNG_ERR_ARG);
-            const int smem = row_ctas(KIND, fmt, false) && threads == kSyncBlock
+            const int smem = alone || (row_ctas(KIND, fmt, false) && threads == kSyncBlock)
                                  ? one_cta_smem((const void *)sync, threads)
                                  : 0;
             sync<<<(unsigned)blocks, threads, smem, st>>>(p.state, p.a, p.n, steps, o, p.ld,
@@ -702,24 +771,27 @@ int launch_kind(int fmt, const GenLaunch &p, cudaStream_t st)
             while (threads > 32 && (groups + (uint64_t)threads * sh.v - 1) /
                                            ((uint64_t)threads * sh.v) < kSMs)
                 threads /= 2;
+            if (even)
+                threads = even;
             uint64_t per_block = (uint64_t)threads * sh.v;
             uint64_t blocks = (groups + per_block - 1) / per_block;
             if (blocks > 0x7FFFFFFFull)
                 return set_error(RNG_ERR_ARG);
             // one CTA per SM only for the shape's own CTA size (small calls
             // halve it above to fill the SMs)
-            const int smem =
-                sh.one && threads == sh.block ? one_cta_smem((const void *)vec, threads) : 0;
+            const int smem = alone || (!even && sh.one && threads == sh.block)
+                                 ? one_cta_smem((const void *)vec, threads)
+                                 : 0;
             vec<<<(unsigned)blocks, threads, smem, st>>>(p.state, p.a, p.n, steps, o, p.ld,
                                                          p.s_begin, count);
         } else {
             // realigned groups plus, when count % 4 != 0, one more CTA for the tail
-            int threads = fit_threads(kSyncBlock, main / 4);
-            const uint64_t per_cta = 31 * (threads / 32) + 1;
+            const int threads = even ? even : sync_threads;
+            const uint64_t per_cta = groups_of(threads, true);
             uint64_t blocks = (main / 4 + per_cta - 1) / per_cta + (count > main ? 1 : 0);
             if (blocks > 0x7FFFFFFFull)
                 return set_error(RNG_ERR_ARG);
-            const int smem = row_ctas(KIND, fmt, true) && threads == kSyncBlock
+            const int smem = alone || (row_ctas(KIND, fmt, true) && threads == kSyncBlock)
                                  ? one_cta_smem((const void *)shift, threads)
                                  : 0;
             shift<<<(unsigned)blocks, threads, smem, st>>>(p.state, p.a, p.n, steps, o, p.ld,

@@ -140,12 +140,16 @@ inline uint64_t split_threads(SplitForm form, uint64_t streams)
 // splitting.  More threads fill more of the device as they are, and the jumps
 // of more segments cost more in all.  (xor128 40,001 x 1000: whole 38, split 50
 // us; 10,001 x 8192: 243 and 86.  XORSHIFT8 54,014 x 5838: whole 362, split
-// 431; 10,001 x 8192: 643 and 200.  KISS 150,001 x 300: whole 29, split 44;
+// 431; 10,001 x 8192: 643 and 200.  Aligned xor128 calls of more than a warp a
+// scheduler, f32: 173,440 x 1813 whole 251, split 189; 255,048 x 1233 210 and 193.  KISS 150,001 x 300: whole 29, split 44;
 // 1001 x 300: 17.6 and 13.4.)
 uint64_t split_min_steps(int kind, SplitForm form, uint64_t threads)
 {
     switch (kind) {
-    case RNG_XOR128: return std::max<uint64_t>(1024, std::min<uint64_t>(2048, threads * 3 / 10));
+    case RNG_XOR128:
+        if (form == SplitForm::kAligned && threads > (uint64_t)kSMs * 128)
+            return 1024;
+        return std::max<uint64_t>(1024, std::min<uint64_t>(2048, threads * 3 / 10));
     case RNG_XORSHIFT8: return std::max<uint64_t>(1024, threads * 3 / 5);
     default: break;
     }
