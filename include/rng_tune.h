@@ -20,7 +20,10 @@ extern "C" {
  * (power of two, 32..512), hint = 1 for streaming (evict-first) stores,
  * 0 for default stores, 2 for rows staged in shared memory and written by
  * TMA bulk copies (32-byte aligned rows only; v and block then unused:
- * CTAs of 256 threads, 1024 streams each).  Applies to later rng_generate calls in this process
+ * CTAs of 256 threads, 1024 streams each).  Calls smaller than the device
+ * shrink the CTAs, and until another shape than the built-in one is set, small
+ * calls and those whose last wave would be nearly empty take one group per
+ * thread and CTAs of a size to suit.  Applies to later rng_generate calls in this process
  * on every device; does not change any output.  Returns 0 or RNG_ERR_ARG. */
 int gbrng_set_launch(int kind, int fmt, int v, int block, int hint);
 int gbrng_get_launch(int kind, int fmt, int *v, int *block, int *hint);
@@ -51,7 +54,8 @@ int gbrng_get_row_ctas(int kind, int fmt, int realigned, int *ctas_per_sm);
  * `log2_rows` is log2 of the fewest rows a segment may have for `kind`
  * (1..30); 0 turns splitting off for the kind.  A split generate call takes
  * as many segments as bring its threads up to 2048 per SM (1024 for a
- * consumer call), each a power-of-two number of rows no smaller than that.
+ * consumer call), each no shorter than that: a power of two rows, or of equal
+ * length where the call has all the threads it wants.
  * Outputs never change. */
 int gbrng_set_split(int kind, int log2_rows);
 int gbrng_get_split(int kind, int *log2_rows);

@@ -77,12 +77,15 @@ struct LaunchShape {
     int block;  // CTA size
     int hint;   // streaming stores
     int one;    // one CTA per SM
+    bool set;   // a caller's own: no rule on sizes changes it
 };
 // The shape for a call of `streams` streams (its size class).
 LaunchShape launch_shape(int kind, int fmt, uint64_t streams);
 // CTAs per SM of the barrier-synced kernels for rows that are not 32-byte
 // aligned (realigned: rows not 16-byte aligned): 1, or 0 for as many as fit.
 int row_ctas(int kind, int fmt, bool realigned);
+// Whether a caller set another value than the built-in one.
+bool row_ctas_set(int kind, int fmt, bool realigned);
 // Dynamic shared memory that keeps `kernel`, launched with `threads`
 // threads, to one CTA per SM: more than half an SM's shared memory (nothing
 // is stored there; the reservation only bars a second CTA).  0 when the
@@ -155,6 +158,9 @@ inline bool needs_jump_tables(int kind) { return kind != RNG_MWC32 && kind != RN
 constexpr int kFmtMixed = 2;
 constexpr uint32_t kFmtEnd = 0xFFFFFFFFu;
 
+// batch.cu: rng_plan_create for a plan that is refilled before it is launched.
+rng_plan_handle plan_create_refilled(const rng_batch_item *items, size_t n_items, int threads,
+                                     int ctas_per_sm);
 // batch.cu: refills a plan (rng_plan_refill) with tiles whose outputs are
 // placed and encoded by output maps (OutMap layout, in host words `maps`;
 // item i's map starts at word map_off[i], its origin a device address), and

@@ -692,7 +692,7 @@ int launch_kind(int fmt, const GenLaunch &p, cudaStream_t st)
     // (two halve the warps), and 16-byte stores (TMA rows come in CTAs of 1024
     // streams).  A single warp holds one group per thread anyway, and the
     // fewest rows are over before it matters.
-    if (count < kSmallCall &&
+    if (!sh.set && count < kSmallCall &&
         (sh.hint == 2 || (sh.v == 2 && count > 128 && p.steps >= 16))) {
         sh.v = 1;
         sh.hint = 0;
@@ -708,15 +708,19 @@ int launch_kind(int fmt, const GenLaunch &p, cudaStream_t st)
     const uint64_t main = count & ~(uint64_t)3;
     const int sync_threads = fit_threads(kSyncBlock, main / 4);
     const int vec_threads = fit_threads(sh.block, main / 4 / sh.v);
-    int even = 0;
-    if (!sectors)
-        even = even_threads(KIND, main / 4, groups_of(sync_threads, !aligned), false, !aligned);
     // KISS with 32-byte rows: FP32 takes CTAs of 128, as many as fit, which even
     // out by themselves, and so do uint32 CTAs of less than 512 threads (311,776
-    // streams: 6.6 TB/s, 5.4 in three even waves)
-    else if (KIND != RNG_KISS || (fmt == RNG_U32 && vec_threads == sh.block))
-        even = even_threads(KIND, main / 4, sh.hint == 2 ? kTmaThreads : sh.v * vec_threads, true,
-                            false);
+    // streams: 6.6 TB/s, 5.4 in three even waves).  A caller's own shape stays.
+    const bool fixed = sectors ? sh.set || (KIND == RNG_KISS &&
+                                            (fmt == RNG_F32 || vec_threads < sh.block))
+                               : row_ctas_set(KIND, fmt, !aligned);
+    int even = 0;
+    if (!fixed)
+        even = even_threads(KIND, main / 4,
+                            !sectors       ? groups_of(sync_threads, !aligned)
+                            : sh.hint == 2 ? kTmaThreads
+                                           : sh.v * vec_threads,
+                            sectors, !aligned);
     const bool alone = even && even_alone(KIND, fmt, !aligned);
     if (even && sectors) {
         sh.v = 1;

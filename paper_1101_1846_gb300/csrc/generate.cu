@@ -44,7 +44,7 @@ struct Shape {
 // stays with TMA (1823 against 1818).  At 2^20 x 1024 only xor128 f32 gains
 // (1609-1614 -> 1717 with V = 2).  As for the barrier-synced kernels, fewer
 // warps writing at once keep each SM's write stream denser.
-Shape g_shape[2][kKinds][2] = {
+constexpr Shape kShape[2][kKinds][2] = {
     {
         {{1, 256, 2, 0}, {2, 512, 1, 0}},  // MWC u32, f32
         {{1, 128, 0, 0}, {2, 512, 1, 1}},  // xor128
@@ -62,6 +62,26 @@ Shape g_shape[2][kKinds][2] = {
         {{2, 256, 1, 0}, {2, 256, 1, 0}},  // KISS_XOR
     },
 };
+// The shapes in use: the ones above, and what callers set instead.
+struct SetShape {
+    Shape shape;
+    bool set;
+};
+SetShape g_set_shape[2][kKinds][2];
+
+Shape &shape_to_set(int size_class, int kind, int fmt)
+{
+    SetShape &s = g_set_shape[size_class][kind][fmt];
+    if (!s.set)
+        s = SetShape{kShape[size_class][kind][fmt], true};
+    return s.shape;
+}
+
+const Shape &shape_in_use(int size_class, int kind, int fmt)
+{
+    const SetShape &s = g_set_shape[size_class][kind][fmt];
+    return s.set ? s.shape : kShape[size_class][kind][fmt];
+}
 constexpr uint64_t kSmallStreams = (uint64_t)1 << 21;
 
 // CTAs per SM of the barrier-synced kernels, [kind][fmt][realigned]: 1 =
@@ -74,7 +94,7 @@ constexpr uint64_t kSmallStreams = (uint64_t)1 << 21;
 // Where the step is cheap, fewer warps writing at once keep the write
 // stream denser; the FP32 forms of xor128 and KISS need the second CTA's
 // warps to cover their arithmetic.  The paper's kinds keep 0 (not measured).
-int g_row_ctas[kKinds][2][2] = {
+constexpr int kRowCtas[kKinds][2][2] = {
     {{1, 1}, {1, 1}},  // MWC u32 (16-byte rows, realigned), f32
     {{1, 1}, {1, 0}},  // xor128
     {{1, 1}, {0, 0}},  // KISS
@@ -82,6 +102,7 @@ int g_row_ctas[kKinds][2][2] = {
     {{0, 0}, {0, 0}},  // XORSHIFT8
     {{0, 0}, {0, 0}},  // KISS_XOR
 };
+int g_row_ctas[kKinds][2][2];  // a caller's: 1 + the value, 0 = the table's
 
 // Fewest rows of a split segment, as log2, per kind (0: never split), and
 // the rows it has when that gives threads enough.  The jump that starts a
@@ -167,13 +188,21 @@ uint64_t split_min_steps(int kind, SplitForm form, uint64_t threads)
 
 LaunchShape launch_shape(int kind, int fmt, uint64_t streams)
 {
-    const Shape s = g_shape[streams < kSmallStreams ? 0 : 1][kind][fmt];
-    return LaunchShape{s.v, s.block, s.hint, s.one};
+    const int size_class = streams < kSmallStreams ? 0 : 1;
+    const Shape s = shape_in_use(size_class, kind, fmt), d = kShape[size_class][kind][fmt];
+    return LaunchShape{s.v, s.block, s.hint, s.one,
+                       s.v != d.v || s.block != d.block || s.hint != d.hint || s.one != d.one};
 }
 
 int row_ctas(int kind, int fmt, bool realigned)
 {
-    return g_row_ctas[kind][fmt][realigned ? 1 : 0];
+    const int set = g_row_ctas[kind][fmt][realigned ? 1 : 0];
+    return set ? set - 1 : kRowCtas[kind][fmt][realigned ? 1 : 0];
+}
+
+bool row_ctas_set(int kind, int fmt, bool realigned)
+{
+    return row_ctas(kind, fmt, realigned) != kRowCtas[kind][fmt][realigned ? 1 : 0];
 }
 
 namespace {
@@ -323,7 +352,7 @@ extern "C" int gbrng_set_row_ctas(int kind, int fmt, int realigned, int ctas_per
     if (kind < 0 || kind >= kKinds || fmt < 0 || fmt > 1 || realigned < 0 || realigned > 1 ||
         ctas_per_sm < 0 || ctas_per_sm > 1)
         return set_error(RNG_ERR_ARG);
-    g_row_ctas[kind][fmt][realigned] = ctas_per_sm;
+    g_row_ctas[kind][fmt][realigned] = 1 + ctas_per_sm;
     return RNG_OK;
 }
 
@@ -333,7 +362,7 @@ extern "C" int gbrng_get_row_ctas(int kind, int fmt, int realigned, int *ctas_pe
     if (kind < 0 || kind >= kKinds || fmt < 0 || fmt > 1 || realigned < 0 || realigned > 1 ||
         !ctas_per_sm)
         return set_error(RNG_ERR_ARG);
-    *ctas_per_sm = g_row_ctas[kind][fmt][realigned];
+    *ctas_per_sm = row_ctas(kind, fmt, realigned != 0);
     return RNG_OK;
 }
 
@@ -345,7 +374,7 @@ extern "C" int gbrng_set_launch_class(int kind, int fmt, int size_class, int v, 
         (v != 1 && v != 2) || block < 32 || block > 512 || (block & (block - 1)) || hint < 0 ||
         hint > 2)
         return set_error(RNG_ERR_ARG);
-    Shape &s = g_shape[size_class][kind][fmt];
+    Shape &s = shape_to_set(size_class, kind, fmt);
     s.v = v;
     s.block = block;
     s.hint = hint;
@@ -358,7 +387,7 @@ extern "C" int gbrng_set_launch_ctas(int kind, int fmt, int size_class, int ctas
     if (kind < 0 || kind >= kKinds || fmt < 0 || fmt > 1 || size_class < 0 || size_class > 1 ||
         ctas_per_sm < 0 || ctas_per_sm > 1)
         return set_error(RNG_ERR_ARG);
-    g_shape[size_class][kind][fmt].one = ctas_per_sm;
+    shape_to_set(size_class, kind, fmt).one = ctas_per_sm;
     return RNG_OK;
 }
 
@@ -368,7 +397,7 @@ extern "C" int gbrng_get_launch_ctas(int kind, int fmt, int size_class, int *cta
     if (kind < 0 || kind >= kKinds || fmt < 0 || fmt > 1 || size_class < 0 || size_class > 1 ||
         !ctas_per_sm)
         return set_error(RNG_ERR_ARG);
-    *ctas_per_sm = g_shape[size_class][kind][fmt].one;
+    *ctas_per_sm = shape_in_use(size_class, kind, fmt).one;
     return RNG_OK;
 }
 
@@ -379,9 +408,9 @@ extern "C" int gbrng_get_launch_class(int kind, int fmt, int size_class, int *v,
     if (kind < 0 || kind >= kKinds || fmt < 0 || fmt > 1 || size_class < 0 || size_class > 1 ||
         !v || !block || !hint)
         return set_error(RNG_ERR_ARG);
-    *v = g_shape[size_class][kind][fmt].v;
-    *block = g_shape[size_class][kind][fmt].block;
-    *hint = g_shape[size_class][kind][fmt].hint;
+    *v = shape_in_use(size_class, kind, fmt).v;
+    *block = shape_in_use(size_class, kind, fmt).block;
+    *hint = shape_in_use(size_class, kind, fmt).hint;
     return RNG_OK;
 }
 

@@ -56,3 +56,27 @@ def test_even_xorshift8_equals_the_oracle(n):
     st = oracle.seed_streams(oracle.XORSHIFT8, None, 9, pick)
     want, _ = oracle.generate(oracle.XORSHIFT8, None, st, rows, oracle.U32)
     assert np.array_equal(got[:, pick], np.asarray(want).view(np.uint32).reshape(rows, -1))
+
+
+def test_a_callers_shape_stays():
+    """A shape and a CTAs-per-SM choice that a caller set are used as they are
+    and, set back, give way to the rule again; outputs never change."""
+    import ctypes
+    lib = capi.lib()
+    n, rows = 360_000, 11
+    want = Generator("kiss", n, 3).generate(rows, "u32")
+    v, block, hint = (ctypes.c_int() for _ in range(3))
+    capi.check(lib.gbrng_get_launch_class(oracle.KISS, 0, 0, v, block, hint))
+    old = (v.value, block.value, hint.value)
+    for shape in ((1, 64, 0), (2, 256, 1), old):
+        capi.check(lib.gbrng_set_launch_class(oracle.KISS, 0, 0, *shape))
+        assert torch.equal(Generator("kiss", n, 3).generate(rows, "u32"), want)
+    for n in (360_004, 360_001):
+        realigned = n % 2
+        want = Generator("kiss", n, 3).generate(rows, "u32")
+        for ctas in (0, 1):
+            capi.check(lib.gbrng_set_row_ctas(oracle.KISS, 0, realigned, ctas))
+            got = ctypes.c_int()
+            capi.check(lib.gbrng_get_row_ctas(oracle.KISS, 0, realigned, got))
+            assert got.value == ctas
+            assert torch.equal(Generator("kiss", n, 3).generate(rows, "u32"), want)
