@@ -167,7 +167,7 @@ int rng_state_words(rng_handle h);
 int rng_generate(rng_handle h, uint64_t n_per_stream, void *out, int fmt);
 /* Few streams with long sequences: when n_streams is too small to fill the
  * device, rng_generate cuts each stream's
- * outputs into segments of 2^l rows (l chosen per kind; gbrng_set_split),
+ * outputs into segments (their length chosen per kind and size; gbrng_set_split),
  * starts every segment from the state jumped ahead to it (rng_jump) and
  * runs the segments side by side; the final state goes through a scratch
  * buffer allocated with the handle.  For MWC32 and KISS the segments' MWC
@@ -175,8 +175,8 @@ int rng_generate(rng_handle h, uint64_t n_per_stream, void *out, int fmt);
  * segment), allocated by the first split call that needs it and grown when
  * a call needs more segments: that call synchronises the device and returns
  * RNG_ERR_OOM if the allocation fails.  A split call captured in a CUDA
- * graph, or whose rows are not 16-byte aligned, never allocates; it powers
- * the multipliers in the kernel instead.
+ * graph, whose rows are not 16-byte aligned, or whose segments are long
+ * never allocates; it powers the multipliers in the kernel instead.
  * The outputs and the state are those of the plain sequence (sequence
  * splitting, Sec. "Parallelizing RNGs"). */
 
@@ -352,10 +352,10 @@ typedef struct rng_plan *rng_plan_handle;
  * (power of two, 32..512; 0 = 512), ctas_per_sm = resident CTAs the
  * persistent grid puts on each SM (1..32; 0 = as many as fit); both 0 = the
  * default shape, the fastest measured on GB300 for what the list holds: CTAs
- * of 512 threads, one per SM, or for few tiles CTAs of 64, two or four per SM
+ * of 512 threads, one per SM, or for few tiles CTAs of 64 or 128, two per SM
  * (a refill of such a plan: CTAs of 512 or 128, one per SM).  With ctas_per_sm = 1 the launch
- * reserves more than half an SM's
- * shared memory (unused) so that no SM takes a second CTA.  Items of the
+ * reserves more than half an SM's shared memory (unused) so that no SM takes
+ * a second CTA.  Items of the
  * same handle must cover disjoint stream ranges (they then run side by
  * side); items with n_per_stream = 0 are
  * skipped.  The plan refers to the handles' device

@@ -214,37 +214,39 @@ constexpr int kDefaultCtas = 1;
 
 // Lists of few tiles end with their longest tile, whose rows follow one
 // another faster the fewer warps its SM runs, and they share the SMs more
-// evenly in small tiles: CTAs of 64 threads, two to an SM where some item is
-// long, four where none is (a short tile waits for its state more than for the
-// pipes).  GB300, us a launch, by tiles of 128 threads (4 x 128 streams):
-//                                                        512 x 1  64 x 2  64 x 4
-//     20: 16 items of up to 1174 streams, 400 rows          56.2    27.4    31.1
-//    357: 216 of up to 2268, 1018                          137.6    64.4    81.0
-//    552: 40 of up to 43,000, 16                            13.2    13.8    11.5
-//    612: 40 of up to 43,000, 250                           52.0    31.3    29.9
-//    622: 462 of up to 1064, 820                           141.3    65.7    82.8
-//   1068: 500 of up to 4000, 1000                          187.8    84.7   111.8
-//   1160: 60 of up to 43,000, 250                           43.8    52.8    40.3
-//   1203: 80 of up to 65,536, 1024                         146.6    97.6   119.2
-//   1740: 512 of up to 8000, 500                           101.3    88.4    81.3
-//   1833: 119 of up to 43,400, 87                           37.5    46.3    33.6
-//   2603: 512 of up to 12,000, 1024                        228.2   226.5   230.9
-//   3666: 200 of up to 65,536, 1024                        312.6   364.2   360.0
-//   8787: 512 of up to 65,536, 1024                        719.4   837.4   819.6
-constexpr int kFewThreads = 64;
-constexpr uint64_t kFewTiles = 13;      // per SM: up to here CTAs of 64 threads
-constexpr uint64_t kFewLongTiles = 8;   // per SM: up to here two of them to an SM,
-constexpr uint64_t kFewLongRows = 384;  // when an item has this many rows
+// evenly in small tiles: with a long item CTAs of 64 threads, two to an SM, or
+// of 128 where those would be many; without one CTAs of 128, two to an SM (a
+// short tile waits for its state more than for the pipes).  CTAs of 64, four to
+// an SM, are up to 10 % faster on short lists, but their tiles, twice as many,
+// cost the host more than that when the plan is made.  GB300, us a launch, by
+// tiles of 128 threads (4 x 128 streams):
+//                                                        512 x 1  64 x 2  128 x 2
+//     20: 16 items of up to 1174 streams, 400 rows          56.2    27.4     35.2
+//    357: 216 of up to 2268, 1018                          137.6    64.4     84.5
+//    552: 40 of up to 43,000, 16                            13.2    13.8     12.4
+//    612: 40 of up to 43,000, 250                           52.0    31.3     33.6
+//    622: 462 of up to 1064, 820                           141.3    65.7     84.2
+//   1068: 500 of up to 4000, 1000                          187.8    84.7    111.0
+//   1160: 60 of up to 43,000, 250                           43.8    52.8     42.0
+//   1203: 80 of up to 65,536, 1024                         146.6    97.6    108.3
+//   1740: 512 of up to 8000, 500                           101.3    88.4     80.4
+//   1833: 119 of up to 43,400, 87                           37.5    46.3     37.0
+//   2603: 512 of up to 12,000, 1024                        228.2   226.5    212.4
+//   3666: 200 of up to 65,536, 1024                        312.6   364.2    328.1
+//   8787: 512 of up to 65,536, 1024                        719.4   837.4    761.4
+constexpr uint64_t kFewTiles = 8;        // per SM
+constexpr uint64_t kFewLongTiles = 13;   // per SM, with an item of kFewLongRows rows
+constexpr uint64_t kFewLongRows = 384;
 struct Shape {
     int threads, ctas_per_sm;
 };
 
 Shape shape_for(uint64_t tiles_of_128, uint64_t longest, int sms)
 {
-    if (tiles_of_128 > kFewTiles * sms)
+    const bool slow = longest >= kFewLongRows;
+    if (tiles_of_128 > (slow ? kFewLongTiles : kFewTiles) * sms)
         return Shape{kDefaultThreads, kDefaultCtas};
-    const bool slow = tiles_of_128 <= kFewLongTiles * sms && longest >= kFewLongRows;
-    return Shape{kFewThreads, slow ? 2 : 4};
+    return slow && tiles_of_128 <= kFewTiles * sms ? Shape{64, 2} : Shape{128, 2};
 }
 
 constexpr int kHint = 1;  // streaming stores, as the plain kernels
@@ -362,15 +364,37 @@ uint64_t fill_units(const rng_batch_item *items, size_t n_items, int threads, Un
 
 // Longest tiles first; ties by generator and first stream, so the order is
 // deterministic (it only affects scheduling).
+bool unit_before(const Unit &x, const Unit &y)
+{
+    if (x.steps != y.steps)
+        return x.steps > y.steps;
+    if (x.state != y.state)
+        return x.state < y.state;
+    return x.s0 != y.s0 ? x.s0 < y.s0 : x.out < y.out;
+}
+
 void order_units(Unit *u, uint64_t n)
 {
-    std::sort(u, u + n, [](const Unit &x, const Unit &y) {
-        if (x.steps != y.steps)
-            return x.steps > y.steps;
-        if (x.state != y.state)
-            return x.state < y.state;
-        return x.s0 != y.s0 ? x.s0 < y.s0 : x.out < y.out;
+    std::sort(u, u + n, unit_before);
+}
+
+// The tiles of `items` in that order.  The items are sorted in place of their
+// tiles, of which there are several each: 4000 tiles of 64 bytes took the host
+// some 200 us to sort.
+std::vector<Unit> ordered_units(const rng_batch_item *items, size_t n_items, int threads)
+{
+    std::vector<rng_batch_item> by(items, items + n_items);
+    std::sort(by.begin(), by.end(), [](const rng_batch_item &x, const rng_batch_item &y) {
+        const Gen *g = reinterpret_cast<Gen *>(x.h), *h = reinterpret_cast<Gen *>(y.h);
+        if (x.n_per_stream != y.n_per_stream)
+            return x.n_per_stream > y.n_per_stream;
+        return g->d_state != h->d_state ? g->d_state < h->d_state : x.s_begin < y.s_begin;
     });
+    std::vector<Unit> units(fill_units(by.data(), n_items, threads, nullptr, 0));
+    fill_units(by.data(), n_items, threads, units.data(), units.size());
+    if (!std::is_sorted(units.begin(), units.end(), unit_before))
+        order_units(units.data(), units.size());
+    return units;
 }
 
 uint64_t longest_of(const rng_batch_item *items, size_t n_items)
@@ -451,6 +475,13 @@ struct Plan {
     uint64_t pinned_maps_cap[2] = {0, 0};
 };
 
+// Places for a refill's n tiles: where lists choose their shape, for as many as
+// the smaller tiles are taken for.
+uint64_t refill_room(const Plan &p, uint64_t n)
+{
+    return std::max<uint64_t>(n, kRefillTiles * p.sms);
+}
+
 void free_plan(Plan *p)
 {
     if (!p)
@@ -474,8 +505,13 @@ void free_plan(Plan *p)
 
 using namespace gbrng;
 
-extern "C" rng_plan_handle rng_plan_create(const rng_batch_item *items, size_t n_items,
-                                           int threads, int ctas_per_sm)
+namespace gbrng {
+namespace {
+
+// rng_plan_create; with `refilled` the list takes the shape of a refill (the
+// caller refills the plan at once).
+rng_plan_handle create_plan(const rng_batch_item *items, size_t n_items, int threads,
+                            int ctas_per_sm, bool refilled)
 {
     if (!items || n_items == 0) {
         set_error(RNG_ERR_ARG);
@@ -497,13 +533,12 @@ extern "C" rng_plan_handle rng_plan_create(const rng_batch_item *items, size_t n
     if (choose) {
         if (cuda_status(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device)))
             return nullptr;
-        const Shape s = choose_shape(items, n_items, sms);
+        const Shape s = refilled ? refill_shape(items, n_items, sms)
+                                 : choose_shape(items, n_items, sms);
         threads = s.threads;
         ctas_per_sm = s.ctas_per_sm;
     }
-    std::vector<Unit> units(fill_units(items, n_items, threads, nullptr, 0));
-    fill_units(items, n_items, threads, units.data(), units.size());
-    order_units(units.data(), units.size());
+    const std::vector<Unit> units = ordered_units(items, n_items, threads);
 
     int prev = -1;
     cudaGetDevice(&prev);
@@ -520,12 +555,14 @@ extern "C" rng_plan_handle rng_plan_create(const rng_batch_item *items, size_t n
         st = grid_for(device, threads, ctas_per_sm, &p->grid);
     }
     if (!st && p->n_units) {
+        // refills of other shapes should not have to grow the list
+        const uint64_t room = refilled ? refill_room(*p, p->n_units) : p->n_units;
         size_t bytes = p->n_units * sizeof(Unit);
-        if (cudaMalloc(&p->d_units, bytes) != cudaSuccess)
+        if (cudaMalloc(&p->d_units, room * sizeof(Unit)) != cudaSuccess)
             st = set_error(RNG_ERR_OOM);
         else
             st = cuda_status(cudaMemcpy(p->d_units, units.data(), bytes, cudaMemcpyHostToDevice));
-        p->cap_units = p->n_units;
+        p->cap_units = room;
     }
     if (!st && cudaMalloc(&p->d_next, sizeof(unsigned long long)) != cudaSuccess)
         st = set_error(RNG_ERR_OOM);
@@ -536,6 +573,22 @@ extern "C" rng_plan_handle rng_plan_create(const rng_batch_item *items, size_t n
         return nullptr;
     }
     return reinterpret_cast<rng_plan_handle>(p);
+}
+
+}  // namespace
+
+rng_plan_handle plan_create_refilled(const rng_batch_item *items, size_t n_items, int threads,
+                                     int ctas_per_sm)
+{
+    return create_plan(items, n_items, threads, ctas_per_sm, true);
+}
+
+}  // namespace gbrng
+
+extern "C" rng_plan_handle rng_plan_create(const rng_batch_item *items, size_t n_items,
+                                           int threads, int ctas_per_sm)
+{
+    return create_plan(items, n_items, threads, ctas_per_sm, false);
 }
 
 extern "C" int rng_plan_launch(rng_plan_handle h, void *cuda_stream)
@@ -648,7 +701,8 @@ int refill(Plan *p, const rng_batch_item *items, size_t n_items, const uint64_t 
     else
         st = cuda_status(cudaEventCreateWithFlags(&p->copied[k], cudaEventDisableTiming));
     if (!st)
-        st = ensure_pinned(&p->pinned[k], &p->pinned_cap[k], n, p->pinned_cap[k ^ 1]);
+        st = ensure_pinned(&p->pinned[k], &p->pinned_cap[k], refill_room(*p, n),
+                           p->pinned_cap[k ^ 1]);
     if (!st)
         st = ensure_device(&p->d_units, &p->cap_units, n, stream);
     std::vector<const uint32_t *> dmaps;
@@ -797,7 +851,7 @@ int noalloc_ctas(const rng_batch_item *items, size_t n_items, uint64_t n_units, 
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
         return 0;  // grid_for reports it
-    const bool slow = n_units <= kFewLongTiles * sms && longest_of(items, n_items) >= kFewLongRows;
+    const bool slow = n_units <= kFewTiles * sms && longest_of(items, n_items) >= kFewLongRows;
     return slow ? 1 : 2;
 }
 

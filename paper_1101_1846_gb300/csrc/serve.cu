@@ -316,8 +316,8 @@ int launch_tick(Server *S, int lane)
         return RNG_OK;
     int st = RNG_OK;
     if (!S->plan[lane]) {
-        S->plan[lane] = rng_plan_create(S->items.data(), S->items.size(), S->plan_threads,
-                                        S->plan_ctas);
+        S->plan[lane] = plan_create_refilled(S->items.data(), S->items.size(), S->plan_threads,
+                                             S->plan_ctas);
         st = S->plan[lane] ? RNG_OK : rng_last_error();
     }
     if (!st)

@@ -59,9 +59,9 @@ def sizes_of(tiles):
 
 
 @pytest.mark.parametrize("per_sm,over,rows,shape", [
-    (0, 30, 383, (64, 4)), (0, 30, 384, (64, 2)),
-    (8, 0, 384, (64, 2)), (8, 1, 384, (64, 4)),
-    (13, 0, 20, (64, 4)), (13, 1, 20, (512, 1))])
+    (0, 30, 383, (128, 2)), (0, 30, 384, (64, 2)),
+    (8, 0, 384, (64, 2)), (8, 1, 384, (128, 2)), (8, 0, 20, (128, 2)), (8, 1, 20, (512, 1)),
+    (13, 0, 384, (128, 2)), (13, 1, 384, (512, 1))])
 def test_shapes_equal_plain_calls(per_sm, over, rows, shape):
     sm = sms()
     x = Lists(sizes_of(per_sm * sm + over))
@@ -75,7 +75,7 @@ def test_refills_choose_their_shape():
     sm = sms()
     x = Lists(sizes_of(13 * sm + 1))
     plan = Plan(x.take(17, range(10)))
-    assert plan.shape == (64, 4 * sm)
+    assert plan.shape == (128, 2 * sm)
     plan.launch()
     x.check()
     for rows, pick, threads in ((127, range(10), 512), (128, range(10), 128), (9, None, 512),
