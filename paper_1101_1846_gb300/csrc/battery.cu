@@ -101,7 +101,7 @@ count_kernel(const uint32_t *__restrict__ u, uint64_t n, uint64_t s_begin, uint6
 // thread); the ranks packed four bits each and the byte counts in shared memory
 // keep it within 64 registers (spilled words went to L2 past the shared memory:
 // 1.24 ms).  At 65536 x 4096 on GB300 the whole battery call took 12.0 ms with
-// those sorts and takes 1.24 ms with this kernel.
+// those sorts and takes 1.16 ms with this kernel.
 // Inputs that are not spread (a bucket of 16 days or more, more than 32
 // candidates) take repeats_by_sorting, so no input costs more than before.
 constexpr int kSampleWarps = 16;
