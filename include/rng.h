@@ -353,12 +353,10 @@ typedef struct rng_plan *rng_plan_handle;
  * persistent grid puts on each SM (1..32; 0 = as many as fit); both 0 = the
  * default shape, the fastest measured on GB300 for what the list holds: CTAs
  * of 512 threads, one per SM, or for few tiles CTAs of 64 or 128, two per SM
- * (a refill of such a plan: CTAs of 512 or 128, one per SM).  With ctas_per_sm = 1 the launch
- * reserves more than half an SM's shared memory (unused) so that no SM takes
- * a second CTA.  Items of the
- * same handle must cover disjoint stream ranges (they then run side by
- * side); items with n_per_stream = 0 are
- * skipped.  The plan refers to the handles' device
+ * (rng_plan_refill may change it).  With ctas_per_sm = 1 the launch reserves
+ * more than half an SM's shared memory (unused) so that no SM takes a second
+ * CTA.  Items of the same handle must cover disjoint stream ranges (they then
+ * run side by side); items with n_per_stream = 0 are skipped.  The plan refers to the handles' device
  * memory and the out pointers: it must not outlive them.  Items must be
  * of the kinds RNG_MWC32, RNG_XOR128 or RNG_KISS (the persistent kernel
  * carries the bodies of those three only, so that the paper's larger-state
@@ -375,15 +373,19 @@ rng_plan_handle rng_plan_create(const rng_batch_item *items, size_t n_items,
  * (no device-side waits).  Outputs and state afterwards are bit-identical to
  * calling rng_generate on each item in turn; launching again continues every
  * stream, like a second rng_generate.  No host synchronisation, so the call
- * can be captured in a CUDA graph and replayed.  Two launches of the same
- * plan must not overlap on the device. */
+ * can be captured in a CUDA graph and replayed: a replay runs the list the
+ * plan then holds, as many tiles as it had when captured.  Two launches of the
+ * same plan must not overlap on the device. */
 int rng_plan_launch(rng_plan_handle p, void *cuda_stream);
 
 /* Replaces the plan's work list with the tiles of a new set of items (same
- * rules as rng_plan_create; the CTA size and grid stay), enqueueing the copy
- * to the device on `cuda_stream`: a later rng_plan_launch on the same stream
- * runs the new list, and a launch still in flight on that stream finishes
- * with the old one.  The tiles keep the items' order (no length ordering),
+ * rules as rng_plan_create), enqueueing the copy to the device on
+ * `cuda_stream`: a later rng_plan_launch on the same stream runs the new list,
+ * and a launch still in flight on that stream finishes with the old one.  The
+ * CTA size and grid stay, except where the plan has the default shape and no
+ * launch of it was captured in a CUDA graph: then the new list chooses CTAs of
+ * 512 or of 128 threads, one per SM.  A captured launch replayed after a refill
+ * of as many tiles runs the new list.  The tiles keep the items' order (no length ordering),
  * so that a serving loop can rebuild a plan every tick cheaply.  Allocates
  * device memory only when the list outgrows every earlier one (after waiting
  * for `cuda_stream`).  The tiles are written to one of two pinned host lists

@@ -453,7 +453,8 @@ struct Plan {
     unsigned long long *d_next = nullptr;
     int threads = kDefaultThreads;
     int grid = 0;
-    int sms = 0;  // the lists choose their shapes; 0 = the caller's holds
+    int sms = 0;  // the lists choose their shapes; 0 = the shape stays (a caller's, or
+                  // one that a captured launch holds)
     std::vector<Claim> claims;       // refill overlap check
     // refill staging: two pinned host lists used in turn, so that the copy
     // to the device is a plain DMA and the call does not wait for it; a
@@ -603,6 +604,14 @@ extern "C" int rng_plan_launch(rng_plan_handle h, void *cuda_stream)
     cudaGetDevice(&prev);
     if (prev != p->device)
         cudaSetDevice(p->device);
+    // A graph replays the launch with this CTA size and grid, so later refills
+    // have to cut their tiles for them.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (p->sms && (cudaStreamIsCapturing(st, &capture) != cudaSuccess ||
+                   capture != cudaStreamCaptureStatusNone)) {
+        cudaGetLastError();  // the launch below reports what is wrong with the stream
+        p->sms = 0;
+    }
     int status = cuda_status(cudaMemsetAsync(p->d_next, 0, sizeof(unsigned long long), st));
     if (!status) {
         const bool one = p->ctas_per_sm == 1;
