@@ -556,8 +556,8 @@ rng_plan_handle create_plan(const rng_batch_item *items, size_t n_items, int thr
         st = grid_for(device, threads, ctas_per_sm, &p->grid);
     }
     if (!st && p->n_units) {
-        // refills of other shapes should not have to grow the list
-        const uint64_t room = refilled ? refill_room(*p, p->n_units) : p->n_units;
+        // refills of other shapes must not have to grow the list
+        const uint64_t room = refill_room(*p, p->n_units);
         size_t bytes = p->n_units * sizeof(Unit);
         if (cudaMalloc(&p->d_units, room * sizeof(Unit)) != cudaSuccess)
             st = set_error(RNG_ERR_OOM);

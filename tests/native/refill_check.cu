@@ -4,6 +4,9 @@
 // what a replay of the captured launch would run.
 // Input: "before rows n_items", then the items' stream counts; before = 1: the
 // plan is refilled once, with the same items, before the launch is captured.
+// before = 2 "rows n_items fewer rows_then" then the counts: no launch is captured
+// and the plan is refilled with the first `fewer` items at rows_then rows each;
+// the records are left out.
 // Output: "shape" and "tiles" of the plan when captured and after the refill,
 // "allocs" of device memory by the refill, then per record that the replay
 // takes "item mode s0 streams new" (streams: how many a CTA of the captured
@@ -92,7 +95,10 @@ int main()
     int before = 0;
     uint64_t rows = 0;
     size_t n_items = 0;
-    if (std::scanf("%d %" SCNu64 " %zu", &before, &rows, &n_items) != 3)
+    size_t fewer = 0;
+    uint64_t rows_then = 0;
+    if (std::scanf("%d %" SCNu64 " %zu", &before, &rows, &n_items) != 3 ||
+        (before == 2 && std::scanf("%zu %" SCNu64, &fewer, &rows_then) != 2))
         return 2;
     std::vector<Gen> gens(n_items);
     // stand-in addresses: a place for every item's output, the new ones above
@@ -113,16 +119,29 @@ int main()
     }
     const auto old_items = items_at(0), new_items = items_at(fresh);
     rng_plan_handle plan = rng_plan_create(old_items.data(), n_items, 0, 0);
-    if (!plan || (before && rng_plan_refill(plan, old_items.data(), n_items, nullptr)))
+    if (!plan || (before == 1 && rng_plan_refill(plan, old_items.data(), n_items, nullptr)))
         return 1;
+    auto report = [&](const Plan &p) {
+        std::printf("shape %d %d tiles %" PRIu64 "\n", p.threads, p.grid, p.n_units);
+    };
+    if (before == 2) {
+        report(*reinterpret_cast<Plan *>(plan));
+        auto items = new_items;
+        items.resize(fewer);
+        for (rng_batch_item &it : items)
+            it.n_per_stream = rows_then;
+        fake::allocs = 0;
+        if (rng_plan_refill(plan, items.data(), items.size(), nullptr))
+            return 1;
+        report(*reinterpret_cast<Plan *>(plan));
+        std::printf("allocs %d\n", fake::allocs);
+        return 0;
+    }
     fake::capturing = true;
     if (rng_plan_launch(plan, nullptr))
         return 1;
     fake::capturing = false;
     const Plan taken = *reinterpret_cast<Plan *>(plan);  // what the capture holds
-    auto report = [&](const Plan &p) {
-        std::printf("shape %d %d tiles %" PRIu64 "\n", p.threads, p.grid, p.n_units);
-    };
     report(taken);
     fake::allocs = 0;
     if (rng_plan_refill(plan, new_items.data(), n_items, nullptr))

@@ -57,3 +57,16 @@ def test_captured_launch_replays_the_new_list(refill_bin, before, rows, sizes):
             assert s0 == at, (i, s0, at)
             at += streams
         assert at == n, (i, at)
+
+
+@pytest.mark.parametrize("rows,sizes,fewer,more_rows", [
+    (256, [65_536] * 12, 5, 400), (20, [512 * 9 * SMS], 1, 400), (17, [512 * 5 * SMS, 7], 2, 130),
+    (1018, [2268] * 216, 216, 20)])
+def test_a_list_that_does_not_outgrow_the_first_allocates_nothing(refill_bin, rows, sizes, fewer,
+                                                                  more_rows):
+    """The first `fewer` items refill a plan that was never captured, with rows
+    of another count: the smaller tiles a refill may choose fit as well."""
+    text = f"2 {rows} {len(sizes)} {fewer} {more_rows}\n" + "\n".join(map(str, sizes)) + "\n"
+    r = subprocess.run([str(refill_bin)], input=text, capture_output=True, text=True, check=True,
+                       timeout=120)
+    assert r.stdout.split("\n")[-2] == "allocs 0", r.stdout
