@@ -174,7 +174,9 @@ int rng_generate(rng_handle h, uint64_t n_per_stream, void *out, int fmt);
  * jumps come from a per-handle table of multipliers (8 bytes per stream and
  * segment), allocated by the first split call that needs it and grown when
  * a call needs more segments: that call synchronises the device and returns
- * RNG_ERR_OOM if the allocation fails.  A split call captured in a CUDA
+ * RNG_ERR_OOM if the allocation fails.  So do up to four calls of a handle
+ * that need it for segments of another length than calls on another stream
+ * did.  A split call captured in a CUDA
  * graph, whose rows are not 16-byte aligned, or whose segments are long
  * never allocates; it powers the multipliers in the kernel instead.
  * The outputs and the state are those of the plain sequence (sequence

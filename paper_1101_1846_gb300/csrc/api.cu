@@ -64,6 +64,8 @@ void free_gen(Gen *g)
     cudaFree(g->d_split);
     cudaFree(g->d_cnt);
     cudaFree(g->d_jmul);
+    if (g->jmul_built)
+        cudaEventDestroy(g->jmul_built);
     for (int i = 0; i < 2; ++i) {
         cudaFree(g->d_stage[i]);
         if (g->stage_ev[i])

@@ -36,6 +36,12 @@ struct Gen {
     uint64_t jmul_rows = 0;       // rows per segment the table was built for (0: none)
     uint32_t jmul_cap = 0;        // segments the table holds
     uint32_t jmul_segs = 0;       // most segments a split call of this handle has
+    // the stream the table was built on, an event after the build, and whether
+    // other streams have read the table since
+    cudaStream_t jmul_stream = nullptr;
+    cudaEvent_t jmul_built = nullptr;
+    bool jmul_shared = false;
+    int jmul_waits = 0;           // rebuilds that waited for other streams' calls
     // staging for rng_generate_host
     void *d_stage[2] = {nullptr, nullptr};
     size_t stage_bytes = 0;
@@ -131,14 +137,16 @@ int launch_jump(Gen *g, uint64_t k, cudaStream_t st);
 // The handle's MWC jump multipliers for `segs` segments of `rows` rows,
 // rebuilt on `st` when `rows` differs from the table's (MWC32 and KISS
 // handles only).  The table is allocated, or grown, when a call needs more
-// segments than it holds (synchronises then; never inside a capture).
+// segments than it holds (synchronises then; never inside a capture).  A
+// rebuild against which other streams' calls may still be reading it waits for
+// them (synchronises then), a few times in a handle's life; after that *table is
+// nullptr in such a call.
 int mwc_jump_table(Gen *g, uint64_t rows, uint64_t segs, cudaStream_t st,
                    const uint64_t **table);
-// The table if it already holds `segs` segments of `rows` rows, else nullptr.
-inline const uint64_t *ready_jump_table(const Gen *g, uint64_t rows, uint64_t segs)
-{
-    return g->jmul_rows == rows && segs <= g->jmul_cap ? g->d_jmul : nullptr;
-}
+// *table: the table, with `st` made to wait for it, if it already holds `segs`
+// segments of `rows` rows, else nullptr.  Never waits on the host.
+int ready_jump_table(Gen *g, uint64_t rows, uint64_t segs, cudaStream_t st,
+                     const uint64_t **table);
 // Most segments a split call on a handle of n streams can have.
 uint32_t split_max_segments(uint64_t n);
 

@@ -661,17 +661,19 @@ int launch_split_shift(int fmt, const GenLaunch &p, cudaStream_t st, bool *done)
                         resident_ctas((const void *)fn, threads, 0), g->jmul_segs, &seg))
         return RNG_OK;
     JumpTables T{};
+    const uint64_t *jmul = nullptr;
     bool table = false;
     int e = needs_jump_tables(KIND) ? jump_tables(&T) : RNG_OK;
     if (!e && mont_table(KIND))
         e = table_allowed(st, &table);
+    if (!e && table)
+        e = ready_jump_table(g, seg.rows, seg.count, st, &jmul);
     if (e)
         return e;
     *done = true;
     fn<<<dim3((unsigned)tiles, (unsigned)seg.count), threads, 0, st>>>(
         p.state, p.a, p.n, (uint32_t)p.steps, (uint32_t)seg.rows, static_cast<uint32_t *>(p.out),
-        p.ld, p.s_begin, count, warps, g->d_split, g->d_cnt,
-        table ? ready_jump_table(g, seg.rows, seg.count) : nullptr, T);
+        p.ld, p.s_begin, count, warps, g->d_split, g->d_cnt, jmul, T);
     return cuda_status(cudaGetLastError());
 }
 

@@ -344,17 +344,58 @@ int jump_tables(JumpTables *out)
     return RNG_OK;
 }
 
+namespace {
+
+constexpr int kMostTableWaits = 4;
+
+// Hands the table to a call on `st`, after its build.
+int use_jump_table(Gen *g, cudaStream_t st, const uint64_t **table)
+{
+    if (st != g->jmul_stream) {
+        const int e = cuda_status(cudaStreamWaitEvent(st, g->jmul_built, 0));
+        if (e)
+            return e;
+        g->jmul_shared = true;
+    }
+    *table = g->d_jmul;
+    return RNG_OK;
+}
+
+}  // namespace
+
+int ready_jump_table(Gen *g, uint64_t rows, uint64_t segs, cudaStream_t st,
+                     const uint64_t **table)
+{
+    *table = nullptr;
+    if (!g->d_jmul || g->jmul_rows != rows || segs > g->jmul_cap)
+        return RNG_OK;
+    return use_jump_table(g, st, table);
+}
+
 int mwc_jump_table(Gen *g, uint64_t rows, uint64_t segs, cudaStream_t st,
                    const uint64_t **table)
 {
     if (!g->d_a || segs == 0 || segs > g->jmul_segs)
         return set_error(RNG_ERR_ARG);
-    if (segs > g->jmul_cap) {
-        // grow: the old table may still be read by earlier calls (on any
-        // stream), so wait for the device before freeing it
-        int e = cuda_status(cudaDeviceSynchronize());
+    const bool grow = segs > g->jmul_cap;
+    if (!grow && g->jmul_rows == rows)
+        return use_jump_table(g, st, table);
+    // The old table may still be read by earlier calls: on this stream they come
+    // before a rebuild, but on another (or before the table is freed) the
+    // device has to finish them.  A handle that keeps changing streams and
+    // lengths goes without the table in the end.
+    const bool wait = g->d_jmul && (g->jmul_shared || st != g->jmul_stream);
+    if (wait && !grow && g->jmul_waits == kMostTableWaits) {
+        *table = nullptr;
+        return RNG_OK;
+    }
+    if (grow || wait) {
+        const int e = cuda_status(cudaDeviceSynchronize());
         if (e)
             return e;
+        g->jmul_waits += wait && !grow ? 1 : 0;
+    }
+    if (grow) {
         cudaFree(g->d_jmul);
         g->d_jmul = nullptr;
         g->jmul_cap = 0;
@@ -363,16 +404,24 @@ int mwc_jump_table(Gen *g, uint64_t rows, uint64_t segs, cudaStream_t st,
             return set_error(RNG_ERR_OOM);
         g->jmul_cap = (uint32_t)segs;
     }
-    if (g->jmul_rows != rows) {
-        const uint64_t total = g->n * g->jmul_cap;
-        const uint64_t blocks = (total + 255) / 256;
-        mwc_table_kernel<<<(unsigned)blocks, 256, 0, st>>>(g->d_a, g->n, rows, g->jmul_cap,
-                                                           g->d_jmul);
-        int e = cuda_status(cudaGetLastError());
-        if (e)
-            return e;
-        g->jmul_rows = rows;
-    }
+    int e = RNG_OK;
+    if (!g->jmul_built)
+        e = cuda_status(cudaEventCreateWithFlags(&g->jmul_built, cudaEventDisableTiming));
+    if (e)
+        return e;
+    const uint64_t total = g->n * g->jmul_cap;
+    const uint64_t blocks = (total + 255) / 256;
+    g->jmul_rows = 0;  // until the new one is on its way
+    mwc_table_kernel<<<(unsigned)blocks, 256, 0, st>>>(g->d_a, g->n, rows, g->jmul_cap,
+                                                       g->d_jmul);
+    g->jmul_stream = st;
+    g->jmul_shared = false;
+    e = cuda_status(cudaGetLastError());
+    if (!e)
+        e = cuda_status(cudaEventRecord(g->jmul_built, st));
+    if (e)
+        return e;
+    g->jmul_rows = rows;
     *table = g->d_jmul;
     return RNG_OK;
 }

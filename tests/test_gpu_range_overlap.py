@@ -26,7 +26,7 @@ def _built():
 N, ROWS, CALLS = 10_000, 2100, 12
 # 16-byte rows of groups whose quarter indexes are first streams of the other
 # range; rows that are not 16-byte aligned
-RANGES = [((4000, 8000), 0), ((1, 2002), 2)]
+RANGES = [((4000, 8000), 0), ((1, 3999), 2)]
 
 
 def outputs():
@@ -50,6 +50,39 @@ def test_disjoint_ranges_on_two_streams(kind):
         for _ in range(CALLS):
             for ((b, e), offset), out in zip(RANGES, want):
                 h.generate_range(b, e, ROWS, out, N, "u32", offset=offset)
+    finally:
+        capi.check(capi.lib().gbrng_set_split(kind, log2.value))
+    torch.cuda.synchronize()
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
+    assert torch.equal(g.get_state(), h.get_state())
+    g.close()
+    h.close()
+
+
+@pytest.mark.parametrize("kind", [oracle.MWC, oracle.KISS])
+def test_jump_table_between_streams(kind):
+    """MWC32 and KISS take the jumps from the handle's table: built by an aligned
+    range's call on one stream, read by an unaligned one's on the other (equal
+    segments), and rebuilt for another length while that may still be running."""
+    log2 = ctypes.c_int()
+    capi.check(capi.lib().gbrng_get_split(kind, ctypes.byref(log2)))
+    g, h = Generator(kind, N, 18), Generator(kind, N, 18)
+    got, want = outputs(), outputs()
+    streams = [torch.cuda.Stream() for _ in RANGES]
+    lengths = [2100, 1500, 2100, 900, 2100, 1500, 1200, 2100, 900, 1500, 2100, 1200]
+
+    def calls(gen, outs, where):
+        for rows in lengths:
+            for ((b, e), offset), out, s in zip(RANGES, outs, where):
+                gen.generate_range(b, e, rows, out, N, "u32", offset=offset, stream=s)
+
+    torch.cuda.synchronize()
+    calls(g, got, streams)
+    torch.cuda.synchronize()
+    capi.check(capi.lib().gbrng_set_split(kind, 0))
+    try:
+        calls(h, want, [None, None])
     finally:
         capi.check(capi.lib().gbrng_set_split(kind, log2.value))
     torch.cuda.synchronize()
