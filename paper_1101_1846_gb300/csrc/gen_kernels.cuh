@@ -690,16 +690,6 @@ int launch_kind(int fmt, const GenLaunch &p, cudaStream_t st)
         return RNG_OK;
     LaunchShape sh = launch_shape(KIND, fmt, count);
     const int split_hint = sh.hint;
-    // The shape is for calls that fill the device.  Below kSmallCall streams
-    // there is less than a CTA of it per SM: one group of four per thread then
-    // (two halve the warps), and 16-byte stores (TMA rows come in CTAs of 1024
-    // streams).  A single warp holds one group per thread anyway, and the
-    // fewest rows are over before it matters.
-    if (!sh.set && count < kSmallCall &&
-        (sh.hint == 2 || (sh.v == 2 && count > 128 && p.steps >= 16))) {
-        sh.v = 1;
-        sh.hint = 0;
-    }
     // 16-byte rows and 16-byte state groups: every group of four streams
     // starts on a 16-byte boundary in the output and in the state words.
     const bool aligned = (count % 4 == 0) && (p.ld % 4 == 0) && ((uintptr_t)p.out % 16 == 0) &&
@@ -708,6 +698,19 @@ int launch_kind(int fmt, const GenLaunch &p, cudaStream_t st)
                          (p.a == nullptr || (uintptr_t)p.a % 16 == 0);
     // whole 32-byte sectors per warp and row: no barriers needed
     const bool sectors = aligned && (p.ld % 8 == 0) && ((uintptr_t)p.out % 32 == 0);
+    // The shape is for calls that fill the device.  Below kSmallCall streams
+    // there is less than a CTA of it per SM: one group of four per thread then
+    // (two halve the warps), and 16-byte stores (TMA rows come in CTAs of 1024
+    // streams).  A single warp holds one group per thread anyway, and the
+    // fewest rows are over before it matters.  The kernels of other rows, which
+    // take only the store hint from the shape, keep it: their form without it is
+    // up to twice as slow (KISS_XOR u32, 20,000 streams x 100 rows from an odd
+    // word, us: 8.2 with streaming stores, 12.3 without).
+    if (sectors && !sh.set && count < kSmallCall &&
+        (sh.hint == 2 || (sh.v == 2 && count > 128 && p.steps >= 16))) {
+        sh.v = 1;
+        sh.hint = 0;
+    }
     const uint64_t main = count & ~(uint64_t)3;
     const int sync_threads = fit_threads(kSyncBlock, main / 4);
     const int vec_threads = fit_threads(sh.block, main / 4 / sh.v);
