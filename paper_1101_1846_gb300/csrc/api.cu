@@ -154,10 +154,10 @@ rng_handle create_range(int kind, uint64_t s_begin, uint64_t n_streams, uint64_t
     if (!st && n_streams <= kSplitMaxStreams) {
         g->jmul_segs = split_max_segments(n_streams);
         if (cudaMalloc(&g->d_split, (size_t)g->words * n_streams * 4) != cudaSuccess ||
-            cudaMalloc(&g->d_cnt, n_streams * 4) != cudaSuccess)
+            cudaMalloc(&g->d_cnt, split_counters(n_streams) * 4) != cudaSuccess)
             st = set_error(RNG_ERR_OOM);
         else
-            st = cuda_status(cudaMemset(g->d_cnt, 0, n_streams * 4));
+            st = cuda_status(cudaMemset(g->d_cnt, 0, split_counters(n_streams) * 4));
     }
     // jump tables of the xorshift and LCG parts, built here so that no later
     // call (which may be captured in a CUDA graph) has to build them

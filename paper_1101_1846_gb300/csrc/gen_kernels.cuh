@@ -114,8 +114,7 @@ constexpr int kShiftSplitWarps = 4;
 //
 // Writing the final state back must wait until every segment has read the
 // start state, and no segment may wait for another.  So each thread counts
-// its arrival on the group's counter, the word of its first stream (calls of
-// disjoint ranges may run side by side), right after reading the start state;
+// its arrival on the group's counter right after reading the start state;
 // the last segment also stashes its final state and counts once more.  The
 // arrival that brings the count to segments + 1 sees every read done and the
 // final state ready: it writes the state (from registers or the stash) and
@@ -168,7 +167,7 @@ gen_split(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult, uint6
     if constexpr (KindTraits<KIND>::MULT)
         load4(mult + s0, a);
     __threadfence();  // the reads above are done before the arrival is counted
-    uint32_t *cnt = counters + s0;
+    uint32_t *cnt = counters + s0 / 4;
     const bool finish = live && atomicAdd(cnt, 1u) == segs;
     if (finish) {
         // every other arrival, the stash included, came first
@@ -673,7 +672,7 @@ int launch_split_shift(int fmt, const GenLaunch &p, cudaStream_t st, bool *done)
     *done = true;
     fn<<<dim3((unsigned)tiles, (unsigned)seg.count), threads, 0, st>>>(
         p.state, p.a, p.n, (uint32_t)p.steps, (uint32_t)seg.rows, static_cast<uint32_t *>(p.out),
-        p.ld, p.s_begin, count, warps, g->d_split, g->d_cnt, jmul, T);
+        p.ld, p.s_begin, count, warps, g->d_split, shift_counters(g), jmul, T);
     return cuda_status(cudaGetLastError());
 }
 
