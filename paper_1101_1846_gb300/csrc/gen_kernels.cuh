@@ -184,6 +184,7 @@ gen_split(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult, uint6
         jump.fill(first, T);
         // MWC32 / KISS: the tabulated a^(y*rows) when the handle's table is
         // passed, else powering (calls captured in a CUDA graph)
+        bool powers = true;
         if constexpr (KIND == RNG_MWC32 || KIND == RNG_KISS) {
             if (jmul) {
                 const uint4 lo =
@@ -193,13 +194,17 @@ gen_split(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult, uint6
                 const uint64_t A[4] = {(uint64_t)lo.y << 32 | lo.x, (uint64_t)lo.w << 32 | lo.z,
                                        (uint64_t)hi.y << 32 | hi.x, (uint64_t)hi.w << 32 | hi.z};
                 mwc_jump_streams<KIND, 4>(w, a, first, A);
-            } else {
-                mwc_jump_streams<KIND, 4>(w, a, first, nullptr);
+                powers = false;
             }
-        } else {
-            mwc_jump_streams<KIND, 4>(w, a, first, nullptr);
         }
-        jump.template apply<4>(w);
+        // not by the threads past the last group: 24 streams x 15,000 rows, us a
+        // call with their powers and without, MWC captured 10.2 and 6.7, MWC16X2
+        // 11.9 and 7.9, KISS_XOR 16.3 and 12.3
+        if (live) {
+            if (powers)
+                mwc_jump_streams<KIND, 4>(w, a, first, nullptr);
+            jump.template apply<4>(w);
+        }
     }
     if (!SYNC && !live)
         return;  // after the CTA's part of the jump
