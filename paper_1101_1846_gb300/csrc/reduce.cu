@@ -18,6 +18,7 @@ namespace gbrng {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr unsigned kOneCtaEach = 152;  // CTAs of which every SM has one
 
 // The next output.  MWC32 steps by a wide product and two carrying adds here:
 // that takes the adds off the FMA-heavy pipe, which bounds its consumers
@@ -52,11 +53,11 @@ __device__ __forceinline__ uint32_t next_of(Engine<KIND> &e)
 }
 
 // A pair (u0, u1) is inside when X^2 + Y^2 < 2^48, X = u0 >> 8, Y = u1 >> 8.
-template <int KIND>
+template <int KIND, bool DISC = true>
 __device__ __forceinline__ uint32_t disc_pair(Engine<KIND> &e)
 {
-    const uint64_t X = next_of<KIND, true>(e) >> 8;
-    const uint64_t Y = next_of<KIND, true>(e) >> 8;
+    const uint64_t X = next_of<KIND, DISC>(e) >> 8;
+    const uint64_t Y = next_of<KIND, DISC>(e) >> 8;
     return (X * X + Y * Y) >> 48 == 0 ? 1u : 0u;
 }
 
@@ -104,7 +105,7 @@ __device__ __forceinline__ uint32_t disc_block(Engine<KIND> &e)
 // kinds were unchanged).  256 values of 24 bits fit 32: their chunks add up
 // in 32 bits, one shifted add per output in place of a shift and a 64-bit
 // add.
-template <int OP, int KIND>
+template <int OP, bool SPLIT, int KIND>
 __device__ __forceinline__ uint64_t consume(Engine<KIND> &e, uint64_t m)
 {
     uint64_t acc = 0;
@@ -131,6 +132,16 @@ __device__ __forceinline__ uint64_t consume(Engine<KIND> &e, uint64_t m)
     } else {
         // kPairs pairs at a time by disc_block, the rest one by one
         uint64_t left = m / 2;
+        if constexpr (KIND == RNG_KISS_XOR && !SPLIT) {
+            // A whole call of this kind (at most 76,636 streams) has few rows;
+            // with at most a CTA per SM it takes the integer test, whose chain is
+            // shorter (us, blocks and pairs: 4 x 198 6.9 and 5.0, 20,000 x 256
+            // 10.8 and 9.0; 76,636 x 256 15.3 and 15.9).
+            if (gridDim.x <= kOneCtaEach)
+#pragma unroll 4
+                for (; left; --left)
+                    acc += disc_pair<KIND, false>(e);
+        }
         for (; left >= kPairs; left -= kPairs)
             acc += disc_block(e);
         for (; left; --left)
@@ -198,7 +209,7 @@ reduce_kernel(rng_device_view v, uint64_t steps, uint64_t rows, uint64_t *__rest
             return;
         Engine<KIND> e;
         e.load(v, s);
-        out[s] = consume<OP>(e, steps);
+        out[s] = consume<OP, SPLIT>(e, steps);
         e.store(v, s);
         return;
     }
@@ -238,7 +249,7 @@ reduce_kernel(rng_device_view v, uint64_t steps, uint64_t rows, uint64_t *__rest
     if (!live)
         return;  // after the CTA's part of the jump
     atomicAdd(reinterpret_cast<unsigned long long *>(out + s),
-              (unsigned long long)consume<OP>(e, mine));
+              (unsigned long long)consume<OP, SPLIT>(e, mine));
     if (blockIdx.y == segs - 1) {
         rng_device_view f = v;
         f.state = stash;
