@@ -106,13 +106,14 @@ int launch_generate_paper(int kind, int fmt, const GenLaunch &p, cudaStream_t st
 int resident_ctas(const void *kernel, int threads, int smem);
 
 // Whether a call that advances `streams` streams `steps` times is split into
-// segments.
+// segments (fmt: its outputs' format; any for a consumer).
 enum class SplitForm {
-    kAligned,  // generate, 16-byte rows: four streams per thread
-    kShifted,  // generate, other rows: four streams per thread
+    kAligned,  // generate, 32-byte rows: four streams per thread
+    kShifted,  // generate, rows not 16-byte aligned: four streams per thread
+    kRows16,   // generate, 16- but not 32-byte rows: four streams per thread
     kReduce    // consumers: one stream per thread
 };
-bool split_wanted(int kind, SplitForm form, uint64_t streams, uint64_t steps);
+bool split_wanted(int kind, SplitForm form, int fmt, uint64_t streams, uint64_t steps);
 // Its segments, for `tiles` CTAs per segment and `resident` CTAs on the device
 // at once (0: unknown).  False when there would be only one.
 struct Segments {

@@ -625,8 +625,8 @@ int launch_split(int fmt, int hint, bool sectors, const GenLaunch &p, cudaStream
     const uint64_t count = p.s_end - p.s_begin, tiles = (count / 4 + 255) / 256;
     const int smem = !sectors && KIND != RNG_KISS_XOR ? kSyncSplitSmem : 0;
     Segments seg;
-    if (!split_segments(KIND, SplitForm::kAligned, count, p.steps, tiles,
-                        resident_ctas((const void *)fn, 256, smem), g->jmul_segs, &seg))
+    if (!split_segments(KIND, sectors ? SplitForm::kAligned : SplitForm::kRows16, count, p.steps,
+                        tiles, resident_ctas((const void *)fn, 256, smem), g->jmul_segs, &seg))
         return RNG_OK;
     JumpTables T{};
     const uint64_t *jmul = nullptr;
@@ -748,8 +748,10 @@ int launch_kind(int fmt, const GenLaunch &p, cudaStream_t st)
     }
     uint32_t *out = static_cast<uint32_t *>(p.out);
     Gen *g = p.owner;
-    const SplitForm form = aligned ? SplitForm::kAligned : SplitForm::kShifted;
-    if (g && g->d_split && split_wanted(KIND, form, count, p.steps)) {
+    const SplitForm form = sectors   ? SplitForm::kAligned
+                           : aligned ? SplitForm::kRows16
+                                     : SplitForm::kShifted;
+    if (g && g->d_split && split_wanted(KIND, form, fmt, count, p.steps)) {
         bool done = false;
         const int e = aligned ? launch_split<KIND>(fmt, split_hint, sectors, p, st, &done)
                               : launch_split_shift<KIND>(fmt, p, st, &done);

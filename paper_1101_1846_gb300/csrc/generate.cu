@@ -157,31 +157,85 @@ inline uint64_t split_threads(SplitForm form, uint64_t streams)
     return form == SplitForm::kReduce ? streams : (streams + 3) / 4;
 }
 
-// Fewest rows of a call of `threads` threads a segment that is worth
-// splitting.  More threads fill more of the device as they are, and the jumps
-// of more segments cost more in all.  (xor128 40,001 x 1000: whole 38, split 50
-// us; 10,001 x 8192: 243 and 86.  XORSHIFT8 54,014 x 5838: whole 362, split
-// 431; 10,001 x 8192: 643 and 200.  Aligned xor128 calls of more than a warp a
-// scheduler, f32: 173,440 x 1813 whole 251, split 189; 255,048 x 1233 210 and 193.  KISS 150,001 x 300: whole 29, split 44;
-// 1001 x 300: 17.6 and 13.4.)
-uint64_t split_min_steps(int kind, SplitForm form, uint64_t threads)
+// Fewest rows of a call that is worth splitting.  More threads fill more of the
+// device as they are, and the jumps of more segments cost more in all.  Timed
+// whole and split on GB300, us:
+//   xor128       40,001 x 1000: 38, 50; 10,001 x 8192: 243, 86; aligned calls of
+//                more than a warp a scheduler, f32: 173,440 x 1813 251, 189;
+//                255,048 x 1233 210, 193
+//   XORSHIFT8    4096 x 1024: 52, 59; 10,001 x 8192: 643, 200; 40,000 x 6000: 302,
+//                272; 50,000 x 8000: 402, 430; x 16,000: 802, 687
+//   MWC          20,000 x 200: 10.4, 8.5; 40,000 x 256: 12.4, 14.5; x 400: 17, 15;
+//                76,632 x 400: 22, 23; x 1000: 49, 47
+//   KISS         20,000 x 129: 10.4, 8.5; 40,000 x 200: 12.6, 14.5; x 300: 18.4,
+//                16.5; 76,632 x 400: 23, 25
+//   MWC16X2      4096 x 160: 8.3, 10.4; x 200: 10.4, 8.5; 40,000 x 500: 20, 23;
+//                x 1300: 45, 39; 76,632 x 1000: 50, 53; x 2000: 99, 97
+//   KISS_XOR     20,000 x 160: 11.4, 12.6; 40,000 x 300: 18.6, 22.7; x 400: 24, 23;
+//                76,632 x 700: 39, 49; 16-byte rows 76,636 x 200: 18.6, 18.7; x 400:
+//                29, 27 (their whole form pays for row barriers)
+uint64_t aligned_min_steps(int kind, bool sectors, uint64_t threads)
 {
-    switch (kind) {
-    case RNG_XOR128:
-        if (form == SplitForm::kAligned && threads > (uint64_t)kSMs * 128)
-            return 1024;
-        return std::max<uint64_t>(1024, std::min<uint64_t>(2048, threads * 3 / 10));
-    case RNG_XORSHIFT8: return std::max<uint64_t>(1024, threads * 3 / 5);
-    default: break;
-    }
     // shorter calls take 4-8 us whole, one group per thread (kSmallCall), and as
     // long split
-    const uint64_t least = 129;
-    if (kind == RNG_KISS_XOR)  // the slowest steps: the whole call takes longest
-        return std::max(least, form == SplitForm::kShifted ? threads / 50 : 0);
+    constexpr uint64_t least = 129;
+    switch (kind) {
+    case RNG_XOR128:
+        return threads > (uint64_t)kSMs * 128
+                   ? 1024
+                   : std::max<uint64_t>(1024, std::min<uint64_t>(2048, threads * 3 / 10));
+    case RNG_XORSHIFT8:
+        return threads > 10000 ? 16000 : std::max<uint64_t>(1150, threads * 3 / 5);
+    case RNG_MWC32: return std::max(least, threads / (sectors ? 40 : 64));
+    case RNG_KISS: return std::max(least, threads / 40);
+    case RNG_MWC16X2: return std::max<uint64_t>(180, threads / (sectors ? 15 : 20));
+    default:
+        if (!sectors)
+            return std::max(least, threads / 60);
+        return std::max<uint64_t>(threads < 1000 ? least : 180,
+                                  threads / (threads <= 14000 ? 28 : 13));
+    }
+}
+
+// The same for rows that are not 16-byte aligned: fewer than four streams, which
+// run one to a thread with no row to realign (three streams, whole and split, us:
+// xor128 u32 x 4000 38, 40, f32 x 3000 38, 35; XORSHIFT8 x 6000 132, 143; KISS u32 x
+// 500 12, 14, f32 x 400 14, 13; MWC x 400 4.6, 4.8; MWC16X2 x 400 5.5, 5.8; KISS_XOR
+// u32 x 500 12.1, 12.7, f32 x 400 13.4, 12.3), one group of four (XORSHIFT8 x 1254
+// 86, 91; KISS u32 x 256 12.5, 13.3; KISS_XOR u32 x 160 11.3, 12.0), or more (KISS
+// 150,001 x 300: 29, 44; 1001 x 300: 17.6, 13.4; KISS_XOR, the slowest steps, 1001 x
+// 129: 14.8, 9.4; XORSHIFT8 54,014 x 5838: 362, 431).
+uint64_t shifted_min_steps(int kind, int fmt, uint64_t streams, uint64_t threads)
+{
+    constexpr uint64_t kTail[2][kKinds] = {{450, 4400, 600, 450, 7000, 560},
+                                           {450, 2800, 380, 450, 7000, 360}};
+    constexpr uint64_t kGroup[2][kKinds] = {{256, 1024, 288, 256, 1300, 200},
+                                            {256, 1024, 256, 256, 1300, 150}};
+    if (streams <= 4)
+        return (streams < 4 ? kTail : kGroup)[fmt == RNG_F32 ? 1 : 0][kind];
+    switch (kind) {
+    case RNG_XOR128:
+        return std::max<uint64_t>(1024, std::min<uint64_t>(2048, threads * 3 / 10));
+    case RNG_XORSHIFT8: return std::max<uint64_t>(1024, threads * 3 / 5);
+    case RNG_KISS_XOR: return std::max<uint64_t>(129, threads / 50);
+    default: return std::max<uint64_t>(256, std::min<uint64_t>(1024, threads / 10));
+    }
+}
+
+uint64_t split_min_steps(int kind, SplitForm form, int fmt, uint64_t streams)
+{
+    const uint64_t threads = split_threads(form, streams);
     if (form == SplitForm::kShifted)
-        return std::max<uint64_t>(256, std::min<uint64_t>(1024, threads / 10));
-    return std::max(least, kind == RNG_MWC16X2 ? threads / 50 : 0);
+        return shifted_min_steps(kind, fmt, streams, threads);
+    if (form != SplitForm::kReduce)
+        return aligned_min_steps(kind, form == SplitForm::kAligned, threads);
+    switch (kind) {
+    case RNG_XOR128:
+        return std::max<uint64_t>(1024, std::min<uint64_t>(2048, threads * 3 / 10));
+    case RNG_XORSHIFT8: return std::max<uint64_t>(1024, threads * 3 / 5);
+    case RNG_MWC16X2: return std::max<uint64_t>(129, threads / 50);
+    default: return 129;
+    }
 }
 
 }  // namespace
@@ -290,14 +344,14 @@ uint32_t split_max_segments(uint64_t n)
     return (uint32_t)std::min<uint64_t>(kSplitFillThreads / std::max<uint64_t>(threads, 1), 65535);
 }
 
-bool split_wanted(int kind, SplitForm form, uint64_t streams, uint64_t steps)
+bool split_wanted(int kind, SplitForm form, int fmt, uint64_t streams, uint64_t steps)
 {
     if (g_split_log2[kind] == 0 || streams == 0 || streams > kSplitMaxStreams ||
         steps > (1ull << 31))
         return false;
     const uint64_t threads = split_threads(form, streams);
     return 2 * threads <= kFewStreamThreads &&  // else they fill the device already
-           steps >= split_min_steps(kind, form, threads);
+           steps >= split_min_steps(kind, form, fmt, streams);
 }
 
 bool split_segments(int kind, SplitForm form, uint64_t streams, uint64_t steps, uint64_t tiles,
