@@ -145,10 +145,13 @@ constexpr uint64_t kFewStreamThreads = (uint64_t)kSMs * 1024;
 constexpr uint64_t kSplitFillThreads = (uint64_t)kSMs * 2048;
 
 // KISS_XOR, whose steps cost most of those with cheap jumps, runs best as one
-// wave of CTAs while its segments stay this short (76,636 x 4096 u32: 195 us in
-// one wave of 512-row segments, 204 in two; 40,004 x 4096 116 and 130; with
-// 1500 rows 590 in one, 545 in more).
-constexpr uint64_t kOneWaveRows = 512;
+// wave of CTAs while its segments stay this short (u32, us in one wave and in
+// more, by rows of the one wave's segments: 512 76,636 x 4096 193, 205; 683
+// 20,004 x 12,288 162, 183; 768 76,636 x 6144 279, 290; 1024 76,636 x 8192 367,
+// 375; 1536 76,636 x 12,288 592, 544.  Realigned rows: 30,001 x 8192, 683 rows,
+// 187, 200, but 76,633 x 4096, 1024 rows, 264, 252).
+constexpr uint64_t kOneWaveRows = 1024;
+constexpr uint64_t kOneWaveRowsShifted = 512;
 
 inline uint64_t round8(uint64_t rows) { return (rows + 7) / 8 * 8; }
 
@@ -364,7 +367,8 @@ bool split_segments(int kind, SplitForm form, uint64_t streams, uint64_t steps, 
         std::min<uint64_t>((reduce ? kFewStreamThreads : kSplitFillThreads) / threads, 65535),
         max_segments);
     if (kind == RNG_KISS_XOR && !reduce && resident >= 2 * tiles &&
-        steps <= kOneWaveRows * (resident / tiles))
+        steps <= (form == SplitForm::kShifted ? kOneWaveRowsShifted : kOneWaveRows) *
+                     (resident / tiles))
         want = std::min(want, resident / tiles);
     if (want < 2)
         return false;
