@@ -95,10 +95,17 @@ gen_shift(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult, uint6
 // Dynamic shared memory (nothing is stored there) that keeps gen_split of 16-
 // but not 32-byte rows to three CTAs of 256 threads per SM: as in the
 // barrier-synced kernels, fewer warps writing at once keep the write stream
-// denser.  76,636 x 4096 on GB300, us a call without it and with it: MWC 221
-// -> 189, KISS 209 -> 191, MWC16X2 194 -> 189 (two per SM: 397, 378 and 395 at
-// 8192 rows, against 377, 382 and 379 with three and 447, 415 and 417 without);
-// KISS_XOR, bound by its arithmetic, keeps as many as fit.
+// denser.  GB300, us a call without it and with it (two per SM: 397, 378 and 395
+// at 76,636 x 8192, against 377, 382 and 379 with three and 447, 415 and 417
+// without, MWC, KISS and MWC16X2):
+//                    MWC u32   f32       KISS u32  MWC16X2 u32  xor128 u32
+//   20,004 x 4096     59  56    58  59    64  62    69  59       84  84
+//   40,004 x 4096    109 105   111 102   110 112   110 103      118 120
+//   60,004 x 8192    323 303   328 299   317 298   325 302      337 329
+//   76,636 x 8192    403 380   417 379   410 386   410 378      397 405
+// KISS f32 is within 2 % either way.  KISS_XOR and XORSHIFT8, bound by their
+// arithmetic, keep as many as fit (XORSHIFT8, of whose CTAs with their 24 KB
+// matrix only two would: f32 40,004 x 16,384 823 797, 10,004 x 8192 224 217).
 constexpr int kSyncSplitSmem = 60 * 1024;
 
 // Warps of groups per CTA of gen_split_shift (125 groups), beside its tail warp.
@@ -623,7 +630,8 @@ int launch_split(int fmt, int hint, bool sectors, const GenLaunch &p, cudaStream
                  : (hint ? gen_split<KIND, RNG_U32, 1, true> : gen_split<KIND, RNG_U32, 0, true>);
     Gen *g = p.owner;
     const uint64_t count = p.s_end - p.s_begin, tiles = (count / 4 + 255) / 256;
-    const int smem = !sectors && KIND != RNG_KISS_XOR ? kSyncSplitSmem : 0;
+    const bool dense = KIND != RNG_KISS_XOR && KIND != RNG_XORSHIFT8;
+    const int smem = !sectors && dense ? kSyncSplitSmem : 0;
     Segments seg;
     if (!split_segments(KIND, sectors ? SplitForm::kAligned : SplitForm::kRows16, count, p.steps,
                         tiles, resident_ctas((const void *)fn, 256, smem), g->jmul_segs, &seg))
