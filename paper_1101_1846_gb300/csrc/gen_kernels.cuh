@@ -514,7 +514,8 @@ constexpr int kSMs = 152;
 // 4096 x 128 u32 on GB300, device time of a whole call in us, two groups per
 // thread (MWC u32 by TMA: 8.6 for 4096 x 64) against one: MWC 8.7 and 5.4 (3.4),
 // KISS 12.9 and 7.3, xor128 9.8 and 4.8, MWC16X2 8.5 and 5.0, KISS_XOR 14.0 and
-// 7.6 (9.9 with streaming stores).
+// 7.6 (9.9 with streaming stores); 4096 x 8: KISS 2.2 and 1.8, MWC16X2 1.9 and
+// 1.7, KISS_XOR 2.2 and 1.9; 65,536 x 2: KISS 1.8 and 1.7, the others the same.
 constexpr uint64_t kSmallCall = (uint64_t)kSMs * 1024;
 // CTA size of the kernels with row barriers: large CTAs leave fewer CTA
 // boundaries, where neighbouring CTAs that drift apart split sectors.
@@ -713,13 +714,12 @@ int launch_kind(int fmt, const GenLaunch &p, cudaStream_t st)
     // The shape is for calls that fill the device.  Below kSmallCall streams
     // there is less than a CTA of it per SM: one group of four per thread then
     // (two halve the warps), and 16-byte stores (TMA rows come in CTAs of 1024
-    // streams).  A single warp holds one group per thread anyway, and the
-    // fewest rows are over before it matters.  The kernels of other rows, which
+    // streams).  A single warp holds one group per thread anyway.  The kernels of other rows, which
     // take only the store hint from the shape, keep it: their form without it is
     // up to twice as slow (KISS_XOR u32, 20,000 streams x 100 rows from an odd
     // word, us: 8.2 with streaming stores, 12.3 without).
     if (sectors && !sh.set && count < kSmallCall &&
-        (sh.hint == 2 || (sh.v == 2 && count > 128 && p.steps >= 16))) {
+        (sh.hint == 2 || (sh.v == 2 && count > 128))) {
         sh.v = 1;
         sh.hint = 0;
     }
