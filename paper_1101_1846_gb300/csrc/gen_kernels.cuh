@@ -534,7 +534,7 @@ inline int fit_threads(int threads, uint64_t units)
 // with its last one, which a fixed CTA size leaves nearly empty: 700,000 streams
 // in CTAs of 4096 are 171 CTAs, and 19 of 152 SMs write the second half.  Where
 // less than kEvenFill of the SMs' time is used, the CTAs are made smaller, equal,
-// and as many as whole waves hold.  Every size from one to thirteen waves was
+// and at most as many as whole waves hold.  Every size from one to thirteen waves was
 // timed both ways; above that fill they differ by a few percent either way.
 // GB300, TB/s, fixed and even sizes (r: realigned rows), fill:
 //   KISS u32    668,784 x 470  0.54  4.58  6.45    191,762r x 1640 0.64  4.45  6.11
@@ -553,34 +553,56 @@ inline uint64_t groups_of(int threads, bool realigned)
     return realigned ? 31 * (threads / 32) + 1 : threads;
 }
 
+// Whether even CTAs keep an SM to themselves (one_cta_smem): the realigned
+// FP32 kernels, whose conversions wait longer, and XORSHIFT8 run faster beside
+// one another.
+inline bool even_alone(int kind, int fmt, bool realigned)
+{
+    return kind != RNG_XORSHIFT8 && !(realigned && fmt == RNG_F32 && kind != RNG_MWC32);
+}
+
 // The CTA size for `groups` groups of four, 0 where CTAs of `per_cta` groups
 // fill their waves.  XORSHIFT8, whose steps take the longest, wants the warps of
 // whole SMs; the others write in denser streams from at most 256 threads, and
 // xor128, whose steps take the shortest, 32-byte rows from 128 (f32 calls of
 // 1.2 GB, TB/s in CTAs of 160-224 and of 96-128: 173,440 streams 4.96 6.07,
 // 195,160 5.68 6.54, 255,048 6.35 6.38).
-inline int even_threads(int kind, uint64_t groups, uint64_t per_cta, bool sectors, bool realigned)
+// tail: one more CTA follows, for the last streams of realigned rows.  Where the
+// others would fill their waves exactly it would run after them, so they leave it
+// a place, unless that puts more warps on a scheduler or they are three waves or
+// more that share their SMs (us without the place and with it: XORSHIFT8 340,321 x
+// 924 363, 246, but 453,409 x 693, 13 warps for 12, 214, 259; xor128 f32 189,537 x
+// 1659 278, 217, but 340,929 x 922, three waves, 222, 239; KISS u32 340,929 x 922
+// 228, 210).
+inline int even_threads(int kind, int fmt, uint64_t groups, uint64_t per_cta, bool sectors,
+                        bool realigned, bool tail)
 {
     const uint64_t ctas = (groups + per_cta - 1) / per_cta;
     const uint64_t waves = (ctas + kSMs - 1) / kSMs;
     if (groups <= (uint64_t)kSMs * 128 ||  // at most one warp a scheduler in any case
         (double)groups >= kEvenFill * (double)(per_cta * kSMs * waves))
         return 0;
-    const int most = kind == RNG_XORSHIFT8 ? 512 : kind == RNG_XOR128 && sectors ? 128 : 256;
+    const uint64_t most =
+        kind == RNG_XORSHIFT8 ? 512 : kind == RNG_XOR128 && sectors ? 128 : 256;
+    auto threads_for = [&](uint64_t places) {
+        const uint64_t each = (groups + places - 1) / places;
+        return std::max<uint64_t>(
+            32, realigned ? 32 * ((each - 1 + 30) / 31) : 32 * ((each + 31) / 32));
+    };
     for (uint64_t k = 1;; ++k) {
-        const uint64_t each = (groups + kSMs * k - 1) / (kSMs * k);
-        const uint64_t threads = realigned ? 32 * ((each - 1 + 30) / 31) : 32 * ((each + 31) / 32);
-        if (threads <= (uint64_t)most)
-            return (int)std::max<uint64_t>(threads, 32);
+        const uint64_t threads = threads_for(kSMs * k);
+        if (threads > most)
+            continue;
+        // the CTA of the last streams, which steps them one to a thread
+        const uint64_t each = groups_of((int)threads, realigned);
+        if (tail && (groups + each - 1) / each == kSMs * k &&
+            (k <= 2 || even_alone(kind, fmt, realigned))) {
+            const uint64_t wider = threads_for(kSMs * k - 1);
+            if (wider <= most && (wider + 127) / 128 == (threads + 127) / 128)
+                return (int)wider;
+        }
+        return (int)threads;
     }
-}
-
-// Whether those CTAs keep an SM to themselves (one_cta_smem): the realigned
-// FP32 kernels, whose conversions wait longer, and XORSHIFT8 run faster beside
-// one another.
-inline bool even_alone(int kind, int fmt, bool realigned)
-{
-    return kind != RNG_XORSHIFT8 && !(realigned && fmt == RNG_F32 && kind != RNG_MWC32);
 }
 
 // V = 2 only for kinds of at most four state words: two groups of the
@@ -734,11 +756,11 @@ int launch_kind(int fmt, const GenLaunch &p, cudaStream_t st)
                                : row_ctas_set(KIND, fmt, !aligned);
     int even = 0;
     if (!fixed)
-        even = even_threads(KIND, main / 4,
+        even = even_threads(KIND, fmt, main / 4,
                             !sectors       ? groups_of(sync_threads, !aligned)
                             : sh.hint == 2 ? kTmaThreads
                                            : sh.v * vec_threads,
-                            sectors, !aligned);
+                            sectors, !aligned, !aligned && count > main);
     const bool alone = even && even_alone(KIND, fmt, !aligned);
     if (even && sectors) {
         sh.v = 1;
