@@ -849,19 +849,29 @@ Unit g_noalloc_host_units[kNoAllocMaxTiles];     // host copy of the work list
 Claim g_noalloc_claims[kNoAllocMaxItems];       // overlap check
 
 // CTAs of 128 threads per SM.  The capacity above fixes the tiles, so the
-// list chooses the grid alone: one where a list of few tiles has a long item,
-// else two.  GB300, us, with one / two / four / as many as fit (tiles):
-//    357: 216 items of up to 2268 streams, 1018 rows    64 /   84 /  136 /  176
-//   1068: 500 of up to 4000, 1000                      103 /  111 /  202 /  331
-//   1833: 119 of up to 43,400, 87                       52 /   37 /   42 /   51
-//   8787: 512 of up to 65,536, 1024                    894 /  761 /  910 / 1137
+// list chooses the grid alone: one where a list of few tiles has a long item and
+// the steps are cheap (uint32 of MWC and xor128) or every tile has an SM to
+// itself, else two.  GB300, us, with one / two / four / as many as fit (tiles):
+//    tiles, list                             MWC u32        KISS u32       KISS f32
+//     35: 16 items of up to 1174 x 400    23  34  54  48  29  39  66  60  39  51  81  72
+//    714: 216 of up to 2268 x 1018       196 238 265 343 253 238 277 352 377 309 314 376
+//    809: 30 of up to 20,000 x 400       107 112 135 158 132 113 139 162 192 144 140 167
+//    871: 462 of up to 1064 x 820        178 193 213 268 244 205 233 268 356 271 297 326
+//   1033: 300 of up to 2500 x 500        152 171 189 219 196 170 193 217 282 222 233 228
+// The three kinds mixed, 871 tiles: 266 211 363 725; 1833 (119 items of up to 43,400
+// x 87): 52 37 42 51; 8787 (512 of up to 65,536 x 1024): 894 761 910 1137.
 int noalloc_ctas(const rng_batch_item *items, size_t n_items, uint64_t n_units, int device)
 {
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
         return 0;  // grid_for reports it
-    const bool slow = n_units <= kFewTiles * sms && longest_of(items, n_items) >= kFewLongRows;
-    return slow ? 1 : 2;
+    if (n_units > kFewTiles * sms || longest_of(items, n_items) < kFewLongRows)
+        return 2;
+    bool cheap = true;
+    for (size_t i = 0; i < n_items; ++i)
+        cheap &= items[i].fmt == RNG_U32 &&
+                 reinterpret_cast<const Gen *>(items[i].h)->kind != RNG_KISS;
+    return cheap || n_units <= (uint64_t)sms ? 1 : 2;
 }
 
 }  // namespace
