@@ -163,9 +163,12 @@ inline uint64_t split_threads(SplitForm form, uint64_t streams)
 // Fewest rows of a call that is worth splitting.  More threads fill more of the
 // device as they are, and the jumps of more segments cost more in all.  Timed
 // whole and split on GB300, us:
-//   xor128       40,001 x 1000: 38, 50; 10,001 x 8192: 243, 86; aligned calls of
-//                more than a warp a scheduler, f32: 173,440 x 1813 251, 189;
-//                255,048 x 1233 210, 193
+//   xor128       64 x 400: 11.5, 9.9, f32 x 300: 11.9, 11.2; 1000 x 700: 19, 19, x
+//                927: 25, 19, f32 x 513: 20, 19, x 927: 35, 20;
+//                16-byte rows 1004 x 600: 20, 20, f32 x 400: 25, 20; 20,000 x 1024:
+//                27, 30, f32 x 600: 23, 20; 40,000 x 1024: 34, 45; 10,001 x 8192: 243,
+//                86; calls of more than a warp a scheduler, f32: 173,440 x 1813
+//                251, 189; 255,048 x 1233 210, 193
 //   XORSHIFT8    4096 x 1024: 52, 59; 10,001 x 8192: 643, 200; 40,000 x 6000: 302,
 //                272; 50,000 x 8000: 402, 430; x 16,000: 802, 687
 //   MWC          20,000 x 200: 10.4, 8.5; 40,000 x 256: 12.4, 14.5; x 400: 17, 15;
@@ -177,16 +180,21 @@ inline uint64_t split_threads(SplitForm form, uint64_t streams)
 //   KISS_XOR     20,000 x 160: 11.4, 12.6; 40,000 x 300: 18.6, 22.7; x 400: 24, 23;
 //                76,632 x 700: 39, 49; 16-byte rows 76,636 x 200: 18.6, 18.7; x 400:
 //                29, 27 (their whole form pays for row barriers)
-uint64_t aligned_min_steps(int kind, bool sectors, uint64_t threads)
+uint64_t aligned_min_steps(int kind, int fmt, bool sectors, uint64_t threads)
 {
     // shorter calls take 4-8 us whole, one group per thread (kSmallCall), and as
     // long split
     constexpr uint64_t least = 129;
     switch (kind) {
     case RNG_XOR128:
-        return threads > (uint64_t)kSMs * 128
-                   ? 1024
-                   : std::max<uint64_t>(1024, std::min<uint64_t>(2048, threads * 3 / 10));
+        if (threads > (uint64_t)kSMs * 128)
+            return 1024;
+        if (threads <= 64)
+            return fmt == RNG_F32 ? 300 : 400;
+        if (threads <= (fmt == RNG_F32 ? 5000 : 3700))
+            return fmt == RNG_F32 ? (sectors ? 520 : 400) : sectors ? 760 : 600;
+        return std::max<uint64_t>(
+            1024, std::min<uint64_t>(2048, fmt == RNG_F32 ? threads / 5 : threads * 3 / 10));
     case RNG_XORSHIFT8:
         return threads > 10000 ? 16000 : std::max<uint64_t>(1150, threads * 3 / 5);
     case RNG_MWC32: return std::max(least, threads / (sectors ? 40 : 64));
@@ -231,7 +239,7 @@ uint64_t split_min_steps(int kind, SplitForm form, int fmt, uint64_t streams)
     if (form == SplitForm::kShifted)
         return shifted_min_steps(kind, fmt, streams, threads);
     if (form != SplitForm::kReduce)
-        return aligned_min_steps(kind, form == SplitForm::kAligned, threads);
+        return aligned_min_steps(kind, fmt, form == SplitForm::kAligned, threads);
     switch (kind) {
     case RNG_XOR128:
         return std::max<uint64_t>(1024, std::min<uint64_t>(2048, threads * 3 / 10));

@@ -39,6 +39,9 @@ def wanted():
     (KISS_XOR, ALIGNED, U32, 4096, 160, 180), (MWC16X2, ALIGNED, U32, 60_000, 500, 1000),
     (MWC16X2, ALIGNED, U32, 64, 160, 180), (KISS, ROWS16, U32, 76_636, 200, 500),
     (MWC, ALIGNED, U32, 76_632, 400, 500),
+    (XOR128, ALIGNED, F32, 14_472, 400, 927), (XOR128, ROWS16, F32, 1004, 300, 400),
+    (XOR128, ALIGNED, U32, 64, 399, 400), (XOR128, ALIGNED, F32, 4, 299, 300),
+    (XOR128, ALIGNED, U32, 1000, 700, 760), (XOR128, ALIGNED, U32, 20_000, 1024, 1500),
     (XORSHIFT8, ALIGNED, U32, 76_632, 12_000, 16_000),
     (XORSHIFT8, ALIGNED, F32, 50_000, 8000, 16_000),
     (XORSHIFT8, ALIGNED, U32, 4096, 1100, 1150)])
