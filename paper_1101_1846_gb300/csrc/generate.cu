@@ -161,45 +161,64 @@ inline uint64_t split_threads(SplitForm form, uint64_t streams)
 }
 
 // Fewest rows of a call that is worth splitting.  More threads fill more of the
-// device as they are, and the jumps of more segments cost more in all.  Timed
-// whole and split on GB300, us:
-//   xor128       64 x 400: 11.5, 9.9, f32 x 300: 11.9, 11.2; 1000 x 700: 19, 19, x
-//                927: 25, 19, f32 x 513: 20, 19, x 927: 35, 20;
-//                16-byte rows 1004 x 600: 20, 20, f32 x 400: 25, 20; 20,000 x 1024:
-//                27, 30, f32 x 600: 23, 20; 40,000 x 1024: 34, 45; 10,001 x 8192: 243,
-//                86; calls of more than a warp a scheduler, f32: 173,440 x 1813
-//                251, 189; 255,048 x 1233 210, 193
-//   XORSHIFT8    4096 x 1024: 52, 59; 10,001 x 8192: 643, 200; 40,000 x 6000: 302,
-//                272; 50,000 x 8000: 402, 430; x 16,000: 802, 687
-//   MWC          20,000 x 200: 10.4, 8.5; 40,000 x 256: 12.4, 14.5; x 400: 17, 15;
-//                76,632 x 400: 22, 23; x 1000: 49, 47
-//   KISS         20,000 x 129: 10.4, 8.5; 40,000 x 200: 12.6, 14.5; x 300: 18.4,
-//                16.5; 76,632 x 400: 23, 25
-//   MWC16X2      4096 x 160: 8.3, 10.4; x 200: 10.4, 8.5; 40,000 x 500: 20, 23;
-//                x 1300: 45, 39; 76,632 x 1000: 50, 53; x 2000: 99, 97
-//   KISS_XOR     20,000 x 160: 11.4, 12.6; 40,000 x 300: 18.6, 22.7; x 400: 24, 23;
-//                76,632 x 700: 39, 49; 16-byte rows 76,636 x 200: 18.6, 18.7; x 400:
-//                29, 27 (their whole form pays for row barriers)
+// device as they are, and the jumps of more segments cost more in all; rows of 16
+// bytes, whose whole form pays for row barriers, and FP32, whose whole forms wait
+// longest for their conversions, split sooner.  The lines come from 3400 calls
+// timed whole and split; split over whole, GB300:
+//   rows            200  300  400  500  650  800 1000 1300 1600 2000 2600
+//   MWC u32
+//     20,000        .86  .70  .64
+//     50,000       1.01 1.00  .95 1.00  .87  .98 1.00  .87
+//     76,632       1.17 1.13 1.02 1.03 1.04 1.00  .95 1.02  .96
+//     202,048      1.10 1.08 1.08 1.01 1.00  .99
+//   KISS u32
+//     50,000       1.14  .90  .83  .96  .79  .81
+//     76,632       1.14 1.11 1.09 1.03 1.06 1.07 1.02  .99  .97
+//     202,048       .90  .91  .88  .85
+//   MWC16X2 u32
+//     20,000       1.25  .99 1.12  .95  .78
+//     50,000       1.22 1.16 1.03 1.26 1.10 1.05 1.02  .96 1.00 1.00  .88
+//     76,632       1.17 1.28 1.07 1.15 1.07 1.14 1.06 1.08 1.03  .98  .95
+//     76,636 f32    .89 1.01  .94  .92  .89  .85
+//   KISS_XOR u32
+//     20,000        .97  .91  .75
+//     50,000       1.28 1.20 1.05 1.14  .90  .84  .99  .80
+//     76,632       1.29 1.39 1.20 1.14 1.21 1.13  .98 1.09 1.16  .97  .94
+//     76,636       1.04 1.08  .94  .84  .92
+//   xor128: 1000 x 700 1.0, x 927 .78, f32 x 513 .98, x 927 .57; 1004 x 600 1.0, f32
+//     x 400 .80; 20,000 x 1024 1.10, f32 x 600 .88; 40,000 x 2000 1.16, f32 1.07;
+//     173,440 x 1813 f32 .75
+//   XORSHIFT8: 4096 x 1024 1.14, x 1300 .87, f32 x 1024 .94; 40,000 x 6000 .90;
+//     50,000 x 8000 1.06, x 16,000 .85, f32 x 8000 .90; 76,632 x 16,000 1.20, x
+//     20,000 1.03
 uint64_t aligned_min_steps(int kind, int fmt, bool sectors, uint64_t threads)
 {
     // shorter calls take 4-8 us whole, one group per thread (kSmallCall), and as
     // long split
     constexpr uint64_t least = 129;
+    const bool f32 = fmt == RNG_F32;
+    const bool many = threads > (uint64_t)kSMs * 128;  // more than a warp a scheduler
     switch (kind) {
     case RNG_XOR128:
-        if (threads > (uint64_t)kSMs * 128)
+        if (many)
             return 1024;
         if (threads <= 64)
-            return fmt == RNG_F32 ? 300 : 400;
-        if (threads <= (fmt == RNG_F32 ? 5000 : 3700))
-            return fmt == RNG_F32 ? (sectors ? 520 : 400) : sectors ? 760 : 600;
+            return f32 ? 300 : 400;
+        if (threads <= (f32 ? 5000 : 3700))
+            return f32 ? (sectors ? 520 : 400) : sectors ? 760 : 600;
         return std::max<uint64_t>(
-            1024, std::min<uint64_t>(2048, fmt == RNG_F32 ? threads / 5 : threads * 3 / 10));
+            1024, std::min<uint64_t>(2048, f32 ? threads * 9 / 40 : threads * 3 / 10));
     case RNG_XORSHIFT8:
-        return threads > 10000 ? 16000 : std::max<uint64_t>(1150, threads * 3 / 5);
-    case RNG_MWC32: return std::max(least, threads / (sectors ? 40 : 64));
-    case RNG_KISS: return std::max(least, threads / 40);
-    case RNG_MWC16X2: return std::max<uint64_t>(180, threads / (sectors ? 15 : 20));
+        if (!f32 && threads > 10000 && threads <= 26000)
+            return threads <= 17000 ? 16000 : 24000;
+        return std::max<uint64_t>(f32 || threads <= 64 ? 1024 : 1150, threads * 3 / 5);
+    case RNG_MWC32:
+        return many ? 250 : std::max(least, threads / (sectors ? 40 : f32 ? 80 : 64));
+    case RNG_KISS: return many ? 160 : std::max(least, threads / (f32 && !sectors ? 80 : 42));
+    case RNG_MWC16X2:
+        if (f32 && !sectors)
+            return threads <= 6000 ? least : std::max<uint64_t>(180, threads / 85);
+        return std::max<uint64_t>(180, threads / (sectors ? 17 : 26));
     default:
         if (!sectors)
             return std::max(least, threads / 60);

@@ -38,12 +38,15 @@ def wanted():
     (KISS_XOR, ROWS16, U32, 76_636, 192, 320), (KISS_XOR, ALIGNED, U32, 76_632, 400, 1600),
     (KISS_XOR, ALIGNED, U32, 4096, 160, 180), (MWC16X2, ALIGNED, U32, 60_000, 500, 1000),
     (MWC16X2, ALIGNED, U32, 64, 160, 180), (KISS, ROWS16, U32, 76_636, 200, 500),
-    (MWC, ALIGNED, U32, 76_632, 400, 500),
+    (MWC, ALIGNED, U32, 76_632, 400, 500), (KISS, ALIGNED, U32, 202_048, 150, 160),
+    (KISS, ROWS16, U32, 202_044, 150, 1156), (MWC, ALIGNED, F32, 90_000, 200, 300),
+    (MWC16X2, ROWS16, F32, 76_636, 200, 497),
     (XOR128, ALIGNED, F32, 14_472, 400, 927), (XOR128, ROWS16, F32, 1004, 300, 400),
     (XOR128, ALIGNED, U32, 64, 399, 400), (XOR128, ALIGNED, F32, 4, 299, 300),
     (XOR128, ALIGNED, U32, 1000, 700, 760), (XOR128, ALIGNED, U32, 20_000, 1024, 1500),
-    (XORSHIFT8, ALIGNED, U32, 76_632, 12_000, 16_000),
-    (XORSHIFT8, ALIGNED, F32, 50_000, 8000, 16_000),
+    (XORSHIFT8, ALIGNED, U32, 76_632, 16_000, 24_000),
+    (XORSHIFT8, ALIGNED, U32, 50_000, 8000, 16_000),
+    (XORSHIFT8, ALIGNED, F32, 8, 1023, 1024),
     (XORSHIFT8, ALIGNED, U32, 4096, 1100, 1150)])
 def test_lines(wanted, kind, form, fmt, streams, whole, split):
     assert not wanted(kind, form, fmt, streams, whole)
