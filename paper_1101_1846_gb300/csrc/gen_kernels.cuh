@@ -189,9 +189,14 @@ gen_split(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult, uint6
     if (y > 0) {
         __shared__ SegmentJump<KIND> jump;
         jump.fill(first, T);
+        // the threads past the last group only help to compose: 24 streams x 15,000
+        // rows, us a call with their powers and without, MWC captured 10.2 and 6.7,
+        // MWC16X2 11.9 and 7.9, KISS_XOR 16.3 and 12.3
+        if (!SYNC && !live)
+            return;
         // MWC32 / KISS: the tabulated a^(y*rows) when the handle's table is
         // passed, else powering (calls captured in a CUDA graph)
-        bool powers = true;
+        bool powers = !SYNC || live;
         if constexpr (KIND == RNG_MWC32 || KIND == RNG_KISS) {
             if (jmul) {
                 const uint4 lo =
@@ -204,17 +209,13 @@ gen_split(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult, uint6
                 powers = false;
             }
         }
-        // not by the threads past the last group: 24 streams x 15,000 rows, us a
-        // call with their powers and without, MWC captured 10.2 and 6.7, MWC16X2
-        // 11.9 and 7.9, KISS_XOR 16.3 and 12.3
-        if (live) {
-            if (powers)
-                mwc_jump_streams<KIND, 4>(w, a, first, nullptr);
+        if (powers)
+            mwc_jump_streams<KIND, 4>(w, a, first, nullptr);
+        if (!SYNC || live)
             jump.template apply<4>(w);
-        }
     }
     if (!SYNC && !live)
-        return;  // after the CTA's part of the jump
+        return;
     uint32_t *row = out + (uint64_t)first * ld + c_first;
     if constexpr (SYNC) {
         for (uint32_t j = 0; j < mine; ++j) {
