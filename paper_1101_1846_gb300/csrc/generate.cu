@@ -187,7 +187,7 @@ inline uint64_t split_threads(SplitForm form, uint64_t streams)
 //     76,636       1.04 1.08  .94  .84  .92
 //   xor128: 1000 x 700 1.0, x 927 .78, f32 x 513 .98, x 927 .57; 1004 x 600 1.0, f32
 //     x 400 .80; 20,000 x 1024 1.10, f32 x 600 .88; 40,000 x 2000 1.16, f32 1.07;
-//     173,440 x 1813 f32 .75
+//     60,004 f32 x 600 1.16, x 800 .97; 173,440 x 1813 f32 .75
 //   XORSHIFT8: 4096 x 1024 1.14, x 1300 .87, f32 x 1024 .94; 40,000 x 6000 .90;
 //     50,000 x 8000 1.06, x 16,000 .85, f32 x 8000 .90; 76,632 x 16,000 1.20, x
 //     20,000 1.03
@@ -206,6 +206,8 @@ uint64_t aligned_min_steps(int kind, int fmt, bool sectors, uint64_t threads)
             return f32 ? 300 : 400;
         if (threads <= (f32 ? 5000 : 3700))
             return f32 ? (sectors ? 520 : 400) : sectors ? 760 : 600;
+        if (f32 && !sectors)
+            return threads <= 10000 ? 520 : 760;
         return std::max<uint64_t>(
             1024, std::min<uint64_t>(2048, f32 ? threads * 9 / 40 : threads * 3 / 10));
     case RNG_XORSHIFT8:
