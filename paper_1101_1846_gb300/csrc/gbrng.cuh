@@ -121,8 +121,8 @@ struct Segments {
     uint64_t count;  // at most max_segments
     bool table;      // MWC32, KISS: worth the handle's table of powers
 };
-bool split_segments(int kind, SplitForm form, uint64_t streams, uint64_t steps, uint64_t tiles,
-                    uint64_t resident, uint64_t max_segments, Segments *out);
+bool split_segments(int kind, SplitForm form, int fmt, uint64_t streams, uint64_t steps,
+                    uint64_t tiles, uint64_t resident, uint64_t max_segments, Segments *out);
 
 // jump.cu: device tables of the GF(2) and affine jumps, built on first use
 // on the current device (synchronises then).

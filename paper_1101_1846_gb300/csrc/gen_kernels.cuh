@@ -657,8 +657,9 @@ int launch_split(int fmt, int hint, bool sectors, const GenLaunch &p, cudaStream
     const bool dense = KIND != RNG_KISS_XOR && KIND != RNG_XORSHIFT8;
     const int smem = !sectors && dense ? kSyncSplitSmem : 0;
     Segments seg;
-    if (!split_segments(KIND, sectors ? SplitForm::kAligned : SplitForm::kRows16, count, p.steps,
-                        tiles, resident_ctas((const void *)fn, 256, smem), g->jmul_segs, &seg))
+    const SplitForm form = sectors ? SplitForm::kAligned : SplitForm::kRows16;
+    if (!split_segments(KIND, form, fmt, count, p.steps, tiles,
+                        resident_ctas((const void *)fn, 256, smem), g->jmul_segs, &seg))
         return RNG_OK;
     JumpTables T{};
     const uint64_t *jmul = nullptr;
@@ -693,7 +694,7 @@ int launch_split_shift(int fmt, const GenLaunch &p, cudaStream_t st, bool *done)
     const uint64_t tiles = warps ? (groups + 31 * warps) / (31 * warps + 1) : 1;
     const int threads = 32 * (warps + (count % 4 ? 1 : 0));
     Segments seg;
-    if (!split_segments(KIND, SplitForm::kShifted, count, p.steps, tiles,
+    if (!split_segments(KIND, SplitForm::kShifted, fmt, count, p.steps, tiles,
                         resident_ctas((const void *)fn, threads, 0), g->jmul_segs, &seg))
         return RNG_OK;
     JumpTables T{};

@@ -113,7 +113,9 @@ int g_row_ctas[kKinds][2][2];  // a caller's: 1 + the value, 0 = the table's
 // any multiple of eight rows (76,636 x 2400 MWC: 113 us with 16 of 152 rows, 121
 // with ten of 256), but for xor128 and XORSHIFT8, whose jumps compose a matrix
 // per set bit of the segment's first row (xor128 there: 124 us with 256 rows,
-// 145 with 200), and the consumers.  Its MWC powers are taken in the kernel:
+// 145 with 200), KISS f32, of which half as many CTAs are resident (aligned, us, equal
+// lengths and powers of two: 116,332 x 1335 123, 114; 64,448 x 3137 138, 129; 193,744
+// x 1030 135, 124), and the consumers.  Its MWC powers are taken in the kernel:
 // against rows that long they cost nothing (76,632 x 4096: MWC 184 us with the
 // handle's table, 181 without; KISS 198 and 192), and calls of many lengths
 // rebuild no table.  Shorter segments keep powers of two and the table (MWC
@@ -386,8 +388,8 @@ bool split_wanted(int kind, SplitForm form, int fmt, uint64_t streams, uint64_t 
            steps >= split_min_steps(kind, form, fmt, streams);
 }
 
-bool split_segments(int kind, SplitForm form, uint64_t streams, uint64_t steps, uint64_t tiles,
-                    uint64_t resident, uint64_t max_segments, Segments *out)
+bool split_segments(int kind, SplitForm form, int fmt, uint64_t streams, uint64_t steps,
+                    uint64_t tiles, uint64_t resident, uint64_t max_segments, Segments *out)
 {
     const bool reduce = form == SplitForm::kReduce;
     const uint64_t threads = split_threads(form, streams);
@@ -408,8 +410,9 @@ bool split_segments(int kind, SplitForm form, uint64_t streams, uint64_t steps, 
         L >>= 1;
     // as many segments as threads allow, each longer than L: of one length
     const bool full = count(L) > want;
-    const bool gf2 = kind == RNG_XOR128 || kind == RNG_XORSHIFT8;
-    if (full && !reduce && !gf2) {
+    const bool pow2 = kind == RNG_XOR128 || kind == RNG_XORSHIFT8 ||
+                      (kind == RNG_KISS && fmt == RNG_F32);
+    if (full && !reduce && !pow2) {
         L = round8(count(want));
         L = round8(count(count(L)));
     }

@@ -310,7 +310,7 @@ extern "C" int rng_generate_reduce(rng_handle h, uint64_t n_per_stream, int op, 
     Segments seg{n_per_stream, 1, false};
     const bool split = g->d_split &&
                        split_wanted(g->kind, SplitForm::kReduce, RNG_U32, g->n, n_per_stream) &&
-                       split_segments(g->kind, SplitForm::kReduce, g->n, n_per_stream,
+                       split_segments(g->kind, SplitForm::kReduce, RNG_U32, g->n, n_per_stream,
                                       (g->n + kThreads - 1) / kThreads, 0, g->jmul_segs, &seg);
     const uint64_t rows = seg.rows, segs = seg.count;
     ReduceFn fn = split ? pick_kind<true>(g->kind, op) : pick_kind<false>(g->kind, op);
