@@ -166,21 +166,20 @@ int rng_state_words(rng_handle h);
  * evaluation". */
 int rng_generate(rng_handle h, uint64_t n_per_stream, void *out, int fmt);
 /* Few streams with long sequences: when n_streams is too small to fill the
- * device, rng_generate cuts each stream's
- * outputs into segments (their length chosen per kind and size; gbrng_set_split),
- * starts every segment from the state jumped ahead to it (rng_jump) and
- * runs the segments side by side; the final state goes through a scratch
- * buffer allocated with the handle.  For MWC32 and KISS the segments' MWC
- * jumps come from a per-handle table of multipliers (8 bytes per stream and
- * segment), allocated by the first split call that needs it and grown when
- * a call needs more segments: that call synchronises the device and returns
- * RNG_ERR_OOM if the allocation fails.  So do up to four calls of a handle
- * that need it for segments of another length than calls on another stream
- * did.  A split call captured in a CUDA
- * graph, whose rows are not 16-byte aligned, or whose segments are long
- * never allocates; it powers the multipliers in the kernel instead.
- * The outputs and the state are those of the plain sequence (sequence
- * splitting, Sec. "Parallelizing RNGs"). */
+ * device, rng_generate cuts each stream's outputs into segments (their length
+ * chosen per kind and size; gbrng_set_split), starts every segment from the
+ * state jumped ahead to it (rng_jump) and runs the segments side by side; the
+ * final state goes through a scratch buffer allocated with the handle.  For
+ * MWC32 and KISS the segments' MWC jumps come from a per-handle table of
+ * multipliers (8 bytes per stream and segment), allocated by the first split
+ * call that needs it and grown when a call needs more segments: that call
+ * synchronises the device and returns RNG_ERR_OOM if the allocation fails.  Up
+ * to four calls in a handle's life also synchronise the device, where a call
+ * needs the table for segments of another length and calls on other streams
+ * have used it.  A split call captured in a CUDA graph, whose rows are not
+ * 16-byte aligned, or whose segments are long never allocates; it powers the
+ * multipliers in the kernel instead.  The outputs and the state are those of
+ * the plain sequence (sequence splitting, Sec. "Parallelizing RNGs"). */
 
 /* Advances only streams [s_begin, s_end) (0 <= s_begin < s_end <= n_streams)
  * n_per_stream times; the other streams keep their state.  Output j of
@@ -246,7 +245,7 @@ int rng_generate_reduce(rng_handle h, uint64_t n_per_stream, int op, void *out);
 
 /* Advances every stream by k steps without computing the outputs in
  * between, in O(log k) work per stream: MWC by modular exponentiation
- * (with p = a 2^32 - 1 and t = a x + c, one step maps t to a t mod p), the
+ * (with p = a 2^32 - 1 and z = x + c 2^32, one step maps z to a z mod p), the
  * xorshift parts by powers of their GF(2) matrices (tables of M^(2^m) built
  * once per device on first use; synchronises then), the LCG by composing
  * its affine map.  The state afterwards equals k single steps.

@@ -21,10 +21,11 @@ extern "C" {
  * 0 for default stores, 2 for rows staged in shared memory and written by
  * TMA bulk copies (32-byte aligned rows only; v and block then unused:
  * CTAs of 256 threads, 1024 streams each).  Calls smaller than the device
- * shrink the CTAs, and until another shape than the built-in one is set, small
+ * shrink the CTAs, and while the shape is the built-in one, set or not, small
  * calls and those whose last wave would be nearly empty take one group per
- * thread and CTAs of a size to suit.  Applies to later rng_generate calls in this process
- * on every device; does not change any output.  Returns 0 or RNG_ERR_ARG. */
+ * thread and CTAs of a size to suit.  Applies to later rng_generate calls in
+ * this process on every device; does not change any output.  Returns 0 or
+ * RNG_ERR_ARG. */
 int gbrng_set_launch(int kind, int fmt, int v, int block, int hint);
 int gbrng_get_launch(int kind, int fmt, int *v, int *block, int *hint);
 
@@ -45,18 +46,21 @@ int gbrng_get_launch_ctas(int kind, int fmt, int size_class, int *ctas_per_sm);
 /* CTAs per SM of the kernels for rows that are 16- but not 32-byte aligned
  * (realigned = 0) and for rows that are not 16-byte aligned (realigned = 1),
  * per (kind, fmt): 1 = one CTA of 512 threads per SM (a shared-memory
- * reservation keeps a second one off the SM), 0 = as many as fit.  Outputs
- * never change.  Returns 0 or RNG_ERR_ARG. */
+ * reservation keeps a second one off the SM), 0 = as many as fit.  While the
+ * value is the built-in one, set or not, calls whose last wave would be nearly
+ * empty take CTAs of another size; the other value holds for every call that
+ * fills the device.  Outputs never change.  Returns 0 or RNG_ERR_ARG. */
 int gbrng_set_row_ctas(int kind, int fmt, int realigned, int ctas_per_sm);
 int gbrng_get_row_ctas(int kind, int fmt, int realigned, int *ctas_per_sm);
 
 /* Sequence splitting of few-stream calls (rng_generate, rng_generate_reduce):
  * `log2_rows` is log2 of the fewest rows a segment may have for `kind`
- * (1..30); 0 turns splitting off for the kind.  A split generate call takes
- * as many segments as bring its threads up to 2048 per SM (1024 for a
- * consumer call), each no shorter than that: a power of two rows, or of equal
- * length where the call has all the threads it wants.
- * Outputs never change. */
+ * (1..30); 0 turns splitting off for the kind.  Calls of fewer rows than a
+ * built-in line (by kind, streams, alignment and format) stay whole whatever
+ * it is.  A segment of a split call has at least that many rows, and more while
+ * the call then still has threads enough (built-in lengths per kind): a power
+ * of two, or an equal share where more segments would exceed 2048 threads per
+ * SM (1024 for a consumer call).  Outputs never change. */
 int gbrng_set_split(int kind, int log2_rows);
 int gbrng_get_split(int kind, int *log2_rows);
 

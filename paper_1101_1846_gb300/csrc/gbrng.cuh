@@ -83,7 +83,7 @@ struct LaunchShape {
     int block;  // CTA size
     int hint;   // streaming stores
     int one;    // one CTA per SM
-    bool set;   // a caller's own: no rule on sizes changes it
+    bool set;   // not the built-in one: no rule on sizes changes it
 };
 // The shape for a call of `streams` streams (its size class).
 LaunchShape launch_shape(int kind, int fmt, uint64_t streams);

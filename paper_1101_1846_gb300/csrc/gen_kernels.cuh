@@ -70,8 +70,8 @@ gen_vec_sync(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult, ui
 
 // The first count & ~3 streams in realigned groups of four, 31K + 1 groups
 // per CTA of K warps (see body_shift); the last CTA of the grid takes the
-// count % 4 tail streams (one per thread), so that they run alongside the
-// rest instead of after it.
+// count % 4 tail streams (one per thread), alongside the CTAs of the last wave
+// where these leave it a place (even_threads sees to that).
 template <int KIND, int FMT, int HINT>
 __global__ void __launch_bounds__(512)
 gen_shift(uint32_t *__restrict__ state, const uint32_t *__restrict__ mult, uint64_t n,

@@ -113,12 +113,12 @@ int g_row_ctas[kKinds][2][2];  // a caller's: 1 + the value, 0 = the table's
 // any multiple of eight rows (76,636 x 2400 MWC: 113 us with 16 of 152 rows, 121
 // with ten of 256), but for xor128 and XORSHIFT8, whose jumps compose a matrix
 // per set bit of the segment's first row (xor128 there: 124 us with 256 rows,
-// 145 with 200), KISS f32, of which half as many CTAs are resident (aligned, us, equal
-// lengths and powers of two: 116,332 x 1335 123, 114; 64,448 x 3137 138, 129; 193,744
-// x 1030 135, 124), and the consumers.  Its MWC powers are taken in the kernel:
-// against rows that long they cost nothing (76,632 x 4096: MWC 184 us with the
-// handle's table, 181 without; KISS 198 and 192), and calls of many lengths
-// rebuild no table.  Shorter segments keep powers of two and the table (MWC
+// 145 with 200), KISS f32, of which half as many CTAs are resident (us, equal
+// lengths and powers of two: 116,332 x 1335 121, 113; 64,448 x 3137 134, 128;
+// 193,744 x 1030 131, 123), and the consumers.  Its MWC powers are taken in the
+// kernel: against rows that long they cost nothing (76,632 x 4096: MWC 184 us
+// with the handle's table, 181 without; KISS u32 198 and 192), and calls of many
+// lengths rebuild no table.  Shorter segments keep powers of two and the table (MWC
 // 4096 x 4096: 15.0 us with it, 18.9 without).
 // From a sweep on GB300 of 32 ... 300,001 streams by 150 ... 16384 rows, every
 // kind, aligned and not, segments of 2^5 ... 2^11 rows and whole calls.

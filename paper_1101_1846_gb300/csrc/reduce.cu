@@ -9,7 +9,7 @@
 //
 // One stream per thread, loaded with coalesced 4-byte accesses across the
 // warp.  Few streams with long sequences are split into segments of 2^l
-// rows (split_plan; grid y = segment) that start from jumped states; their
+// rows (split_segments; grid y = segment) that start from jumped states; their
 // results are added into out with 64-bit atomics (exact, in any order), and
 // the final state is written back by the last arrival, as in gen_split.
 #include "jump.cuh"
