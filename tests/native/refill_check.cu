@@ -92,6 +92,8 @@ extern "C" int rng_last_error(void) { return 0; }
 int main()
 {
     using namespace gbrng;
+    // the launches name host memory: they must not find a GPU
+    setenv("CUDA_VISIBLE_DEVICES", "", 1);
     int before = 0;
     uint64_t rows = 0;
     size_t n_items = 0;
