@@ -36,9 +36,10 @@ struct Gen {
     uint64_t jmul_rows = 0;       // rows per segment the table was built for (0: none)
     uint32_t jmul_cap = 0;        // segments the table holds
     uint32_t jmul_segs = 0;       // most segments a split call of this handle has
-    // the stream the table was built on, an event after the build, and whether
+    // the stream the table was built on (its id: a later stream may have the
+    // handle of one that was destroyed), an event after the build, and whether
     // other streams have read the table since
-    cudaStream_t jmul_stream = nullptr;
+    unsigned long long jmul_stream = 0;
     cudaEvent_t jmul_built = nullptr;
     bool jmul_shared = false;
     int jmul_waits = 0;           // rebuilds that waited for other streams' calls

@@ -351,8 +351,12 @@ constexpr int kMostTableWaits = 4;
 // Hands the table to a call on `st`, after its build.
 int use_jump_table(Gen *g, cudaStream_t st, const uint64_t **table)
 {
-    if (st != g->jmul_stream) {
-        const int e = cuda_status(cudaStreamWaitEvent(st, g->jmul_built, 0));
+    unsigned long long id = 0;
+    int e = cuda_status(cudaStreamGetId(st, &id));
+    if (e)
+        return e;
+    if (id != g->jmul_stream) {
+        e = cuda_status(cudaStreamWaitEvent(st, g->jmul_built, 0));
         if (e)
             return e;
         g->jmul_shared = true;
@@ -384,13 +388,17 @@ int mwc_jump_table(Gen *g, uint64_t rows, uint64_t segs, cudaStream_t st,
     // before a rebuild, but on another (or before the table is freed) the
     // device has to finish them.  A handle that keeps changing streams and
     // lengths goes without the table in the end.
-    const bool wait = g->d_jmul && (g->jmul_shared || st != g->jmul_stream);
+    unsigned long long id = 0;
+    int e = cuda_status(cudaStreamGetId(st, &id));
+    if (e)
+        return e;
+    const bool wait = g->d_jmul && (g->jmul_shared || id != g->jmul_stream);
     if (wait && !grow && g->jmul_waits == kMostTableWaits) {
         *table = nullptr;
         return RNG_OK;
     }
     if (grow || wait) {
-        const int e = cuda_status(cudaDeviceSynchronize());
+        e = cuda_status(cudaDeviceSynchronize());
         if (e)
             return e;
         g->jmul_waits += wait && !grow ? 1 : 0;
@@ -404,7 +412,6 @@ int mwc_jump_table(Gen *g, uint64_t rows, uint64_t segs, cudaStream_t st,
             return set_error(RNG_ERR_OOM);
         g->jmul_cap = (uint32_t)segs;
     }
-    int e = RNG_OK;
     if (!g->jmul_built)
         e = cuda_status(cudaEventCreateWithFlags(&g->jmul_built, cudaEventDisableTiming));
     if (e)
@@ -414,7 +421,7 @@ int mwc_jump_table(Gen *g, uint64_t rows, uint64_t segs, cudaStream_t st,
     g->jmul_rows = 0;  // until the new one is on its way
     mwc_table_kernel<<<(unsigned)blocks, 256, 0, st>>>(g->d_a, g->n, rows, g->jmul_cap,
                                                        g->d_jmul);
-    g->jmul_stream = st;
+    g->jmul_stream = id;
     g->jmul_shared = false;
     e = cuda_status(cudaGetLastError());
     if (!e)
