@@ -539,7 +539,7 @@ inline int fit_threads(int threads, uint64_t units)
 // timed both ways; above that fill they differ by a few percent either way.
 // GB300, TB/s, fixed and even sizes (r: realigned rows), fill:
 //   KISS u32    668,784 x 470  0.54  4.58  6.45    191,762r x 1640 0.64  4.45  6.11
-//   KISS f32    200,090r x 1572 0.67 3.87  5.67    373,321r x 842  0.62  3.97  5.16
+//   KISS f32    200,090r x 1572 0.67 3.87  5.82    373,321r x 842  0.62  3.97  5.16
 //   xor128 u32   96,528 x 162  0.62  3.42  4.26    177,530r x 1771 0.59  4.15  6.21
 //   xor128 f32  663,488 x 474  0.53  4.46  7.08    348,553r x 902  0.58  4.06  5.29
 //   XORSHIFT8   197,272 x 1594 0.63  4.29  5.69    338,148r x 930  0.56  3.74  5.01
