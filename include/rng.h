@@ -352,13 +352,16 @@ typedef struct rng_plan *rng_plan_handle;
  * the work list is copied to the device (synchronises).  threads = CTA size
  * (power of two, 32..512; 0 = 512), ctas_per_sm = resident CTAs the
  * persistent grid puts on each SM (1..32; 0 = as many as fit); both 0 = the
- * default shape, the fastest measured on GB300 for what the list holds: CTAs
- * of 512 threads, one per SM, or for few tiles CTAs of 64 or 128, two per SM
- * (rng_plan_refill may change it).  With ctas_per_sm = 1 the launch reserves
- * more than half an SM's shared memory (unused) so that no SM takes a second
- * CTA.  Items of the same handle must cover disjoint stream ranges (they then
- * run side by side); items with n_per_stream = 0 are skipped.  The plan refers to the handles' device
- * memory and the out pointers: it must not outlive them.  Items must be
+ * default shape, the fastest measured on GB300 for what the list holds while
+ * it has the GPU to itself: CTAs of 512 threads, one per SM, or for few tiles
+ * CTAs of 64 or 128, two per SM (rng_plan_refill may change it).  Of lists that
+ * run side by side on two streams, those of more than about three tiles of 512
+ * streams per SM run faster with 512 and 1.  With ctas_per_sm = 1 the launch
+ * reserves more than half an SM's shared memory (unused) so that no SM takes a
+ * second CTA.  Items of the same handle must cover disjoint stream ranges (they
+ * then run side by side); items with n_per_stream = 0 are skipped.  The plan
+ * refers to the handles' device memory and the out pointers: it must not outlive
+ * them.  Items must be
  * of the kinds RNG_MWC32, RNG_XOR128 or RNG_KISS (the persistent kernel
  * carries the bodies of those three only, so that the paper's larger-state
  * variants do not cost the common case registers).  Returns NULL with
